@@ -906,6 +906,8 @@ pq_status layer_fused_impl(const void* q_dev, const void* w_packed_dev, const pq
   }
   const int grid = static_cast<int>(std::min<int64_t>(sms, p.items));
   if (grid <= 0) return PQ_OK;
+  p.items_per_cta = p.items / grid;
+  p.items_rem = p.items % grid;
   CUtensorMap map;
   std::memset(&map, 0, sizeof(map));
   p.pdl = 1;  // programmatic dependent launch: the set-up overlaps the previous grid's last CTAs

@@ -72,7 +72,11 @@ struct Item {
 __device__ __forceinline__ Item item_begin(const ConvParams& p, int64_t it) {
   Item r;
   r.it = it;
-  const int64_t unit = it / p.tiles;
+  // 32-bit division wherever the item count allows it: a 64-bit one is a call of
+  // over a hundred instructions in front of the first load.
+  const int64_t unit = p.items <= 0x7fffffffLL
+                           ? static_cast<int64_t>(static_cast<uint32_t>(it) / static_cast<uint32_t>(p.tiles))
+                           : it / p.tiles;
   r.unit = static_cast<int>(unit);
   r.tile = static_cast<int>(it - unit * p.tiles);
   r.g = r.unit / p.NB;
@@ -81,6 +85,22 @@ __device__ __forceinline__ Item item_begin(const ConvParams& p, int64_t it) {
   r.rb = r.tile - r.n * p.tiles_per_img;
   return r;
 }
+
+// The item's fields are in registers here: the divisions and parameter loads behind
+// them are not moved past a later wait.
+__device__ __forceinline__ void pin(Item& r) {
+  asm volatile("" : "+r"(r.unit), "+r"(r.tile), "+r"(r.g), "+r"(r.nb), "+r"(r.n), "+r"(r.rb));
+}
+
+// Programmatic dependent launch: every global access of a role comes after this
+// wait for the previous kernel on the stream (which may have produced this launch's
+// inputs or may still read its outputs), so stream order holds.  Each role takes it
+// itself, after its own set-up: the parameter loads (cold constant-cache lines, a few
+// hundred cycles each) and divisions in front of a role's loop, 3000 to 3900 cycles
+// before the first load when they followed the wait, then overlap that kernel's end
+// (back to back: 128x28x28, 8 groups of 64, FP4 codes 35.9 -> 34.3 us; the network at
+// batch 1, 20 such layers, 227 -> 216 us).
+__device__ __forceinline__ void wait_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ void item_next(const ConvParams& p, Item& r) {
   ++r.it;
@@ -146,6 +166,8 @@ __device__ __forceinline__ void producer_role(const ConvParams& p, const CUtenso
   const bool a_tma = p.a_tma != 0, flat = p.mode == kModeFlat;
   bool ok = true;
   Item item = item_begin(p, it0);
+  pin(item);
+  if (p.pdl && !p.pdl_early_loads) wait_previous_grid();
   for (int64_t it = it0; it < it1 && ok; ++it, item_next(p, item)) {
     const int64_t unit = item.unit;
     if (p.b_resident && unit != cur_unit) {
@@ -306,6 +328,8 @@ __device__ __forceinline__ void loader_role(const ConvParams& p, const Bars& bar
   bool ok = true;
   const int nph = flat ? 1 : p.nph, Hd = flat ? 1 : p.Hd;
   Item item = item_begin(p, it0);
+  pin(item);
+  if (p.pdl && !p.pdl_early_loads) wait_previous_grid();
   for (int64_t it = it0; it < it1 && ok; ++it, item_next(p, item)) {
     for (int kb = 0; kb < p.n_kb; ++kb) {
       if (!warp_wait(bars.a_empty(ra.stage), ra.phase ^ 1u, ctx)) { ok = false; break; }
@@ -543,8 +567,8 @@ __device__ __forceinline__ void mma_role(const ConvParams& p, const Bars& bars, 
 #pragma unroll
   for (int t = 0; t < kUnrollTaps; ++t) tap_reg[t] = t < taps ? tap_a16[t] : 0u;
   int unit = -1;
-  int tile = static_cast<int>(it0 % tiles);
-  int unit_next = static_cast<int>(it0 / tiles);
+  const Item first = item_begin(p, it0);
+  int tile = first.tile, unit_next = first.unit;
   bool ok = true;
   for (int64_t it = it0; it < it1 && ok; ++it) {
     const int cur = unit_next;
@@ -1131,6 +1155,15 @@ __device__ __forceinline__ void epilogue_role(const ConvParams& p, const Bars& b
   float g_m_out512 = 0.0f, g_m_req512 = 0.0f, g_m_req = 0.0f, g_m_req15 = 0.0f;
   const uint32_t qmax2 = static_cast<uint32_t>(p.qmax_out) * 0x00010001u;
   Item item = item_begin(p, it0);
+  pin(item);
+  if (p.pdl) {
+    wait_previous_grid();
+    // Let the next dependent launch on the stream start its CTAs as SMs free up, but
+    // only once this CTA's own wait has returned: a launch that depends on this one
+    // then starts only after the kernel before this one has completed, so an early
+    // loader two launches on never reads what that kernel is still writing.
+    if (ew == 0 && lane == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
   for (int64_t it = it0; it < it1; ++it, item_next(p, item)) {
     if (item.g != cur_g) {
       cur_g = item.g;
@@ -1342,26 +1375,16 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     tc_fence_after();
   }
 
-  // A programmatic dependent launch: the set-up above (barriers, tensor memory,
-  // scale factors) overlaps the previous grid's last CTAs; every global read and
-  // write below waits for that grid to complete (it may produce this launch's
-  // inputs or read its outputs), so stream order holds.  Where the caller has
-  // promised that the previous kernel writes neither the activations nor the
-  // weights (pdl_early_loads), only the epilogue warps wait: the others' global
-  // accesses are those loads (the producer's copies, the loader warps' reads),
-  // and the quantiser and MMA warps work in shared and tensor memory.
-  const bool third_epi = p.a_tma && !p.a_unpack && !p.a_quant && !p.a_split;  // warps 2-5 run the epilogue too
-  const bool epi_warp = warp >= kFirstEpiWarp || (third_epi && warp >= kFirstLoadWarp);
-  if (p.pdl && (epi_warp || !p.pdl_early_loads)) asm volatile("griddepcontrol.wait;" ::: "memory");
-  // Let the next dependent launch on the stream start its CTAs as SMs free up, but
-  // only once this CTA's own wait has returned: a launch that depends on this one
-  // then starts only after the kernel before this one has completed, so an early
-  // loader two launches on never reads what that kernel is still writing.  The
-  // signal comes from a thread that waited (the first epilogue warp's lane 0).
-  const int first_epi_warp = third_epi ? kFirstLoadWarp : kFirstEpiWarp;
-  if (p.pdl && threadIdx.x == 32 * first_epi_warp) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int64_t it0 = static_cast<int64_t>(blockIdx.x) * p.items / gridDim.x;
-  const int64_t it1 = static_cast<int64_t>(blockIdx.x + 1) * p.items / gridDim.x;
+  // A programmatic dependent launch: the set-up above and each role's own overlap the
+  // previous grid's last CTAs; a role waits for that grid right before its first global
+  // access (wait_previous_grid): the copy role and the loader warps (unless the caller
+  // has promised that the previous kernel writes neither the activations nor the
+  // weights, pdl_early_loads) and the epilogue warps, which make every global store.
+  // The MMA, quantiser, split and unpack roles work in shared and tensor memory only.
+  // a contiguous range of items, sizes differing by at most one
+  const int64_t bx = static_cast<int64_t>(blockIdx.x);
+  const int64_t it0 = bx * p.items_per_cta + min(bx, p.items_rem);
+  const int64_t it1 = it0 + p.items_per_cta + (bx < p.items_rem ? 1 : 0);
   const uint32_t a_base = base;
   const uint32_t b_base = base + p.smem_b_off;
 

@@ -99,6 +99,7 @@ struct ConvParams {
   int tiles_per_img;      // rows mode
   int64_t tiles;          // tiles per (group, n-block) unit
   int64_t items;          // tiles * G * NB
+  int64_t items_per_cta, items_rem;  // items / grid and items % grid: the first items_rem CTAs take one more
   int NB, Nblk, Npow2;    // output-channel blocks, MMA N, TMEM column stride per accumulator
   int MT;                 // 128-row accumulators per tile
   int KC, n_kb, nch;      // channels per K block, K blocks, 16-byte chunks per K block
