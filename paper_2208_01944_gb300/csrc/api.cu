@@ -494,6 +494,8 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
   p.b_unit_bytes = static_cast<uint32_t>(unit_bytes);
   p.lbo_b = static_cast<uint32_t>(p.Nblk) * 16u;
   p.b_stages = resident ? 1 : b_stages;
+  // Two MMA warps in turn where each ring's stages alternate between them for good.
+  p.mma_warps = resident && p.acc_stages == 2 && a_stages % (2 * p.n_kb) == 0 ? 2 : 1;
   {
     const int acc_cols = std::max(32, p.acc_stages * p.MT * p.Npow2);
     p.sf_col = static_cast<uint32_t>(round_up(acc_cols, 32));  // FP4 scale factors after the accumulators

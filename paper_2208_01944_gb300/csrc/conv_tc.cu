@@ -533,7 +533,16 @@ constexpr int kUnrollTaps = 9;
 template <int KSTEPS, int MT, bool F4>
 __device__ __forceinline__ void mma_role(const ConvParams& p, const Bars& bars, uint32_t a_base, uint32_t b_base,
                                          uint32_t tmem_base, const uint32_t* tap_a16, int64_t it0, int64_t it1,
-                                         const WaitCtx& ctx) {
+                                         int mw, const WaitCtx& ctx) {
+  // Two MMA warps (p.mma_warps = 2, on different schedulers) take the items in turn:
+  // warp mw the items it0 + mw, it0 + mw + 2, ...  An item costs its warp about 900
+  // cycles besides its MMAs (commits, the accumulator and operand waits, each slowed
+  // by the epilogue warps of its scheduler), which then pass while the other warp's
+  // MMAs run.  The planner pairs them only where every stage of the operand and
+  // accumulator rings always serves the same warp (a wait on a phase parity cannot
+  // tell a phase from the next but one) and the weights stay in shared memory; both
+  // warps follow every unit's weights, so that neither misses a phase of theirs.
+  //
   // The issue loop must stay lean: the whole warp runs it converged and one
   // elected lane issues each MMA; every extra instruction, branch or
   // long-latency load per MMA lowers tensor-core throughput directly, the more
@@ -569,6 +578,12 @@ __device__ __forceinline__ void mma_role(const ConvParams& p, const Bars& bars, 
   int unit = -1;
   const Item first = item_begin(p, it0);
   int tile = first.tile, unit_next = first.unit;
+  const int n_mw = p.mma_warps;
+  auto skip_item = [&]() {  // the other warp's item
+    racc.advance();
+    for (int kb = 0; kb < n_kb; ++kb) ra.advance();
+  };
+  int turn = mw;  // items until this warp's next one
   bool ok = true;
   for (int64_t it = it0; it < it1 && ok; ++it) {
     const int cur = unit_next;
@@ -580,6 +595,17 @@ __device__ __forceinline__ void mma_role(const ConvParams& p, const Bars& bars, 
       if (!warp_wait(bars.b_full(rb.stage), rb.phase, ctx)) { ok = false; break; }
       unit = cur;
     }
+    const bool unit_ends = resident && (it + 1 >= it1 || unit_next != cur);
+    if (turn > 0) {
+      --turn;
+      skip_item();
+      if (unit_ends) {
+        tc_commit_warp(bars.b_empty(rb.stage));
+        rb.advance();
+      }
+      continue;
+    }
+    turn = n_mw - 1;
     if (!warp_wait(bars.acc_empty(racc.stage), racc.phase ^ 1u, ctx)) { ok = false; break; }
     tc_fence_after();
     const uint32_t d0 = tmem_base + racc.stage * static_cast<uint32_t>(MT) * npow2;
@@ -652,7 +678,7 @@ __device__ __forceinline__ void mma_role(const ConvParams& p, const Bars& bars, 
     if (!ok) break;
     tc_commit_warp(bars.acc_full(racc.stage));
     racc.advance();
-    if (resident && (it + 1 >= it1 || unit_next != cur)) {
+    if (unit_ends) {
       tc_commit_warp(bars.b_empty(rb.stage));
       rb.advance();
     }
@@ -667,10 +693,10 @@ __device__ __forceinline__ void mma_role(const ConvParams& p, const Bars& bars, 
 template <bool F4>
 __device__ __forceinline__ void mma_role_dispatch(const ConvParams& p, const Bars& bars, uint32_t a_base, uint32_t b_base,
                                                   uint32_t tmem_base, const uint32_t* tap_a16, int64_t it0, int64_t it1,
-                                                  const WaitCtx& ctx) {
+                                                  int mw, const WaitCtx& ctx) {
   const int ks = p.nch >> 1;  // one MMA takes 32 bytes of K: 32 FP8 or 64 FP4 channels
 #define PQ_MMA_CASE(K, M) \
-  if (ks == K && p.MT == M) return mma_role<K, M, F4>(p, bars, a_base, b_base, tmem_base, tap_a16, it0, it1, ctx);
+  if (ks == K && p.MT == M) return mma_role<K, M, F4>(p, bars, a_base, b_base, tmem_base, tap_a16, it0, it1, mw, ctx);
   PQ_MMA_CASE(1, 1) PQ_MMA_CASE(1, 2) PQ_MMA_CASE(1, 3) PQ_MMA_CASE(1, 4)
   PQ_MMA_CASE(2, 1) PQ_MMA_CASE(2, 2) PQ_MMA_CASE(2, 3) PQ_MMA_CASE(2, 4)
   PQ_MMA_CASE(3, 1) PQ_MMA_CASE(3, 2) PQ_MMA_CASE(3, 3) PQ_MMA_CASE(3, 4)
@@ -1345,14 +1371,14 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     }
     for (int s = 0; s < bars.B; ++s) {
       mbar_init(bars.b_full(s), 1);
-      mbar_init(bars.b_empty(s), 1);
+      mbar_init(bars.b_empty(s), p.mma_warps);
     }
     for (int s = 0; s < p.acc_stages; ++s) {
       mbar_init(bars.acc_full(s), 1);
       mbar_init(bars.acc_empty(s),
                 (p.a_tma && !p.a_unpack && !p.a_quant && !p.a_split) ? kEpiWarps + kLoadWarps : kEpiWarps);  // one per warp
     }
-    mbar_init(bars.drain(), 1);
+    mbar_init(bars.drain(), p.mma_warps);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -1395,9 +1421,11 @@ __global__ void __launch_bounds__(kConvThreads, 1)
                     WaitCtx{abort_flag, p.err, p.wait_limit_ns, PQ_ERR_PRODUCER});
     }
     __syncwarp();
-  } else if (warp == 1) {
-    mma_role_dispatch<F4>(p, bars, a_base, b_base, tmem_base, tap_a16, it0, it1,
-                      WaitCtx{abort_flag, p.err, p.wait_limit_ns, PQ_ERR_MMA});
+  } else if (warp == 1 || warp == kMma2Warp) {
+    const int mw = __shfl_sync(0xffffffffu, warp == 1 ? 0 : 1, 0);  // warp-uniform for the issue loop
+    if (mw < p.mma_warps)
+      mma_role_dispatch<F4>(p, bars, a_base, b_base, tmem_base, tap_a16, it0, it1, mw,
+                        WaitCtx{abort_flag, p.err, p.wait_limit_ns, PQ_ERR_MMA});
     __syncwarp();
   } else if (warp < kFirstEpiWarp && !p.a_tma) {
     loader_role(p, bars, a_base, it0, it1, WaitCtx{abort_flag, p.err, p.wait_limit_ns, PQ_ERR_PRODUCER});

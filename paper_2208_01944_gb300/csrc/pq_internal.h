@@ -25,7 +25,8 @@ constexpr int kEpiWarps = 4 * kEpiGroups;
 constexpr int kLoadWarps = 4;                      // activation-operand copy warps
 constexpr int kFirstLoadWarp = 2;
 constexpr int kFirstEpiWarp = kFirstLoadWarp + kLoadWarps;
-constexpr int kConvThreads = 32 * (kFirstEpiWarp + kEpiWarps);  // warp 0 weights, 1 MMA, 2-5 loads, 6-13 epilogue
+constexpr int kMma2Warp = kFirstEpiWarp + kEpiWarps;  // the second MMA warp
+constexpr int kConvThreads = 32 * (kMma2Warp + 1);    // warp 0 weights, 1 and 14 MMA, 2-5 loads, 6-13 epilogue
 constexpr int kMaxSmem = 227 * 1024;
 
 enum ConvMode : int { kModeFlat = 0, kModeRows = 1 };
@@ -119,6 +120,7 @@ struct ConvParams {
   uint32_t lbo_b;         // Nblk * 16
   int b_stages;           // ring stages when streamed
   int acc_stages;         // TMEM accumulator buffers (ring of 1..kMaxAccStages)
+  int mma_warps;          // 2: two MMA warps take the items in turn (see mma_role)
   uint32_t tmem_cols;
   uint32_t smem_b_off, smem_stage_off, smem_bar_off, smem_bytes;
   uint32_t stage_q_pitch, stage_f_pitch, stage_warp_bytes;
