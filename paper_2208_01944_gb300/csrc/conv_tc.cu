@@ -164,102 +164,111 @@ __device__ __forceinline__ void producer_role(const ConvParams& p, const CUtenso
   int64_t a_issued = 0, b_issued = 0;
   int64_t cur_unit = -1;
   const bool a_tma = p.a_tma != 0, flat = p.mode == kModeFlat;
+  // Packed codes, fp32 activations and stride-2 windows go to the staging ring, whose
+  // stages the copy warps work into the operand stages.
+  const bool staged = p.a_unpack || p.a_quant || p.a_split;
   bool ok = true;
   Item item = item_begin(p, it0);
   pin(item);
   if (p.pdl && !p.pdl_early_loads) wait_previous_grid();
-  for (int64_t it = it0; it < it1 && ok; ++it, item_next(p, item)) {
-    const int64_t unit = item.unit;
-    if (p.b_resident && unit != cur_unit) {
-      if (!mbar_wait(bars.b_empty(rb.stage), rb.phase ^ 1u, ctx)) break;
-      const uint32_t bar = bars.b_full(rb.stage);
-      mbar_arrive_expect_tx(bar, p.b_unit_bytes);
-      const uint8_t* src = p.w_packed + static_cast<size_t>(unit) * p.b_unit_bytes;
-      for (uint32_t off = 0; off < p.b_unit_bytes; off += 65536u)
-        bulk_load(b_base + off, src + off, min(65536u, p.b_unit_bytes - off), bar);
-      rb.advance();
-      ++b_issued;
-      cur_unit = unit;
-    }
-    if (!a_tma && p.b_resident) continue;
-    for (int kb = 0; kb < p.n_kb && ok; ++kb) {
-      if (a_tma && p.a_quant) {
-        // fp32 activations: a box of 32 channels (one 128-byte swizzled row per
-        // position) into the staging ring; the copy warps quantise it.
-        if (!mbar_wait(bars.pk_empty(ra.stage), ra.phase ^ 1u, ctx)) { ok = false; break; }
-        const uint32_t full = bars.pk_full(ra.stage);
-        mbar_arrive_expect_tx(full, p.a_tx_bytes);
-        const uint32_t dst = pk_base + ra.stage * p.pk_stage_bytes;
-        const int ch0 = p.src_group[item.g] * p.Cin_g + kb * p.KC;
-        // one box per 32 channels of the K block, each on a 1024-byte swizzle atom
-        for (int b = 0; b < (p.KC >> 5); ++b) {
-          const uint32_t db = dst + static_cast<uint32_t>(b) * p.q_box_bytes;
-          if (flat)
-            tma_load_3d(db, tmA, ch0 + 32 * b, item.rb * p.flat_box, item.n, full);
-          else
-            tma_load_4d(db, tmA, ch0 + 32 * b, p.w_coord, item.oh0(p.Ht) + p.h_off, item.n, full);
-        }
-        ra.advance();
-        ++a_issued;
-      } else if (a_tma && p.a_split) {
-        // Stride 2: the tile's whole input window (both stride phases of its rows
-        // and columns) into the staging ring; the copy warps split it into the
-        // phase planes.
-        if (!mbar_wait(bars.pk_empty(ra.stage), ra.phase ^ 1u, ctx)) { ok = false; break; }
-        const uint32_t full = bars.pk_full(ra.stage);
-        mbar_arrive_expect_tx(full, p.a_tx_bytes);
-        const int chi = (p.src_group[item.g] * p.Cin_g + kb * p.KC) >> p.chunk_shift;
-        tma_load_4d(pk_base + ra.stage * p.pk_stage_bytes, tmA, 4 * p.w_coord, 2 * (item.oh0(p.Ht) + p.h_off), chi,
-                    item.n, full);
-        ra.advance();
-        ++a_issued;
-      } else if (a_tma && p.a_unpack) {
-        // Packed codes: the box of 32-bit words into the staging ring; the copy
-        // warps unpack it into the operand stage.
-        if (!mbar_wait(bars.pk_empty(ra.stage), ra.phase ^ 1u, ctx)) { ok = false; break; }
-        const uint32_t full = bars.pk_full(ra.stage);
-        mbar_arrive_expect_tx(full, p.a_tx_bytes);
-        const uint32_t dst = pk_base + ra.stage * p.pk_stage_bytes;
-        const int chi = (p.src_group[item.g] * p.Cin_g + kb * p.KC) >> 4;
+  // The next activation K block to load (K block a_kb of a_item) into stage ra.stage,
+  // once that stage is free (a_slot, parity ra.phase ^ 1).
+  Item a_item = item;
+  int a_kb = 0;
+  int64_t a_left = a_tma ? (it1 - it0) * p.n_kb : 0;
+  auto a_slot = [&]() { return staged ? bars.pk_empty(ra.stage) : bars.a_empty(ra.stage); };
+  auto load_a = [&]() {
+    const uint32_t full = staged ? bars.pk_full(ra.stage) : bars.a_full(ra.stage);
+    mbar_arrive_expect_tx(full, p.a_tx_bytes);
+    const uint32_t dst = staged ? pk_base + ra.stage * p.pk_stage_bytes : a_base + ra.stage * p.a_stage_bytes;
+    const int ch0 = p.src_group[a_item.g] * p.Cin_g + a_kb * p.KC;
+    const int oh0 = a_item.oh0(p.Ht);
+    if (p.a_quant) {
+      // fp32 activations: one box per 32 channels of the K block (one 128-byte
+      // swizzled row per position), each on a 1024-byte swizzle atom
+      for (int b = 0; b < (p.KC >> 5); ++b) {
+        const uint32_t db = dst + static_cast<uint32_t>(b) * p.q_box_bytes;
         if (flat)
-          tma_load_3d(dst, tmA, item.rb * p.flat_box, chi, item.n, full);
+          tma_load_3d(db, tmA, ch0 + 32 * b, a_item.rb * p.flat_box, a_item.n, full);
         else
-          tma_load_4d(dst, tmA, p.w_coord - p.pk_off, item.oh0(p.Ht) + p.h_off, chi, item.n, full);
-        ra.advance();
-        ++a_issued;
-      } else if (a_tma) {
-        if (!mbar_wait(bars.a_empty(ra.stage), ra.phase ^ 1u, ctx)) { ok = false; break; }
-        const uint32_t full = bars.a_full(ra.stage);
-        mbar_arrive_expect_tx(full, p.a_tx_bytes);
-        const uint32_t dst = a_base + ra.stage * p.a_stage_bytes;
-        const int chi = (p.src_group[item.g] * p.Cin_g + kb * p.KC) >> p.chunk_shift;
-        if (flat) {
-          // one box of 128 positions per accumulator, each into its own region
-          for (int mt = 0; mt < p.MT; ++mt)
-            tma_load_3d(dst + static_cast<uint32_t>(mt) * (p.a_mt16 << 4), tmA, 2 * (item.rb * p.flat_box + mt * 128),
-                        chi, item.n, full);
-        } else {
-          tma_load_4d(dst, tmA, 2 * p.w_coord, item.oh0(p.Ht) + p.h_off, chi, item.n, full);
-        }
-        ra.advance();
-        ++a_issued;
+          tma_load_4d(db, tmA, ch0 + 32 * b, p.w_coord, oh0 + p.h_off, a_item.n, full);
       }
-      if (p.b_resident) continue;
-      for (int t = 0; t < p.taps; ++t) {
-        if (!mbar_wait(bars.b_empty(rb.stage), rb.phase ^ 1u, ctx)) { ok = false; break; }
+    } else if (p.a_split) {
+      // Stride 2: the tile's whole input window (both stride phases of its rows
+      // and columns)
+      tma_load_4d(dst, tmA, 4 * p.w_coord, 2 * (oh0 + p.h_off), ch0 >> p.chunk_shift, a_item.n, full);
+    } else if (p.a_unpack) {
+      // Packed codes: the box of 32-bit words
+      if (flat)
+        tma_load_3d(dst, tmA, a_item.rb * p.flat_box, ch0 >> 4, a_item.n, full);
+      else
+        tma_load_4d(dst, tmA, p.w_coord - p.pk_off, oh0 + p.h_off, ch0 >> 4, a_item.n, full);
+    } else if (flat) {
+      // one box of 128 positions per accumulator, each into its own region
+      for (int mt = 0; mt < p.MT; ++mt)
+        tma_load_3d(dst + static_cast<uint32_t>(mt) * (p.a_mt16 << 4), tmA, 2 * (a_item.rb * p.flat_box + mt * 128),
+                    ch0 >> p.chunk_shift, a_item.n, full);
+    } else {
+      tma_load_4d(dst, tmA, 2 * p.w_coord, oh0 + p.h_off, ch0 >> p.chunk_shift, a_item.n, full);
+    }
+    ra.advance();
+    ++a_issued;
+    --a_left;
+    if (++a_kb == p.n_kb) {
+      a_kb = 0;
+      item_next(p, a_item);
+    }
+  };
+  if (p.b_resident) {
+    for (int64_t it = it0; it < it1 && ok; ++it, item_next(p, item)) {
+      const int64_t unit = item.unit;
+      if (unit != cur_unit) {
+        if (!mbar_wait(bars.b_empty(rb.stage), rb.phase ^ 1u, ctx)) break;
         const uint32_t bar = bars.b_full(rb.stage);
-        mbar_arrive_expect_tx(bar, p.b_slice_bytes);
-        const size_t slice = (static_cast<size_t>(unit) * p.taps + t) * p.n_kb + kb;  // tap-major packing
-        bulk_load(b_base + rb.stage * p.b_slice_bytes, p.w_packed + slice * p.b_slice_bytes, p.b_slice_bytes, bar);
+        mbar_arrive_expect_tx(bar, p.b_unit_bytes);
+        const uint8_t* src = p.w_packed + static_cast<size_t>(unit) * p.b_unit_bytes;
+        for (uint32_t off = 0; off < p.b_unit_bytes; off += 65536u)
+          bulk_load(b_base + off, src + off, min(65536u, p.b_unit_bytes - off), bar);
         rb.advance();
         ++b_issued;
+        cur_unit = unit;
+      }
+      for (int kb = 0; a_tma && kb < p.n_kb; ++kb) {
+        if (!mbar_wait(a_slot(), ra.phase ^ 1u, ctx)) { ok = false; break; }
+        load_a();
+      }
+    }
+  } else {
+    // Streamed weights: the next K block's activations are loaded between this
+    // block's weight slices, as soon as their stage is free, so that the block's first
+    // MMA waits for its weights only.  (Loaded right before its weights, a block's
+    // activations arrived 430 to 1000 cycles after the previous block's last MMA:
+    // 128x28x28, 2 groups of 256, 4-bit codes, 87 -> 81 us.)
+    int64_t block = 0;  // K blocks whose weights are issued
+    for (int64_t it = it0; it < it1 && ok; ++it, item_next(p, item)) {
+      const int64_t unit = item.unit;
+      for (int kb = 0; kb < p.n_kb && ok; ++kb, ++block) {
+        if (a_tma && a_issued <= block) {
+          if (!mbar_wait(a_slot(), ra.phase ^ 1u, ctx)) { ok = false; break; }
+          load_a();
+        }
+        for (int t = 0; t < p.taps; ++t) {
+          if (!mbar_wait(bars.b_empty(rb.stage), rb.phase ^ 1u, ctx)) { ok = false; break; }
+          const uint32_t bar = bars.b_full(rb.stage);
+          mbar_arrive_expect_tx(bar, p.b_slice_bytes);
+          const size_t slice = (static_cast<size_t>(unit) * p.taps + t) * p.n_kb + kb;  // tap-major packing
+          bulk_load(b_base + rb.stage * p.b_slice_bytes, p.w_packed + slice * p.b_slice_bytes, p.b_slice_bytes, bar);
+          rb.advance();
+          ++b_issued;
+          if (a_left > 0 && a_issued <= block + 1 && mbar_test(a_slot(), ra.phase ^ 1u)) load_a();
+        }
       }
     }
   }
   // Drain: the last min(stages, issued) copies of each ring may still be in flight.
   const int64_t na = p.a_stages, nbs = p.b_resident ? 1 : p.b_stages;
   for (int64_t k = (a_issued > na ? a_issued - na : 0); k < a_issued; ++k)
-    mbar_wait_drain((p.a_unpack || p.a_quant || p.a_split) ? bars.pk_full(static_cast<int>(k % na)) : bars.a_full(static_cast<int>(k % na)),
+    mbar_wait_drain(staged ? bars.pk_full(static_cast<int>(k % na)) : bars.a_full(static_cast<int>(k % na)),
                     static_cast<uint32_t>((k / na) & 1), ctx.limit_ns, ctx.err);
   for (int64_t k = (b_issued > nbs ? b_issued - nbs : 0); k < b_issued; ++k)
     mbar_wait_drain(bars.b_full(static_cast<int>(k % nbs)), static_cast<uint32_t>((k / nbs) & 1), ctx.limit_ns, ctx.err);
