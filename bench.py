@@ -146,10 +146,10 @@ def source_sha(files):
 
 
 KERNEL_SOURCES = {
-    "pq_conv_tc_kernel<quantise-on-load>": ["conv_tc.cu", "pq_device.cuh", "pq_internal.h"],
+    "pq_conv_tc_kernel<quantise-on-load>": ["conv_tc.cuh", "pq_device.cuh", "pq_internal.h"],
     "pq_quantize_c16": ["quantize.cu", "pq_device.cuh", "pq_internal.h"],
-    "pq_conv_tc_kernel": ["conv_tc.cu", "pq_device.cuh", "pq_internal.h"],
-    "pq_conv_tc_kernel<FP4, quantise-on-load>": ["conv_tc.cu", "pq_device.cuh", "pq_internal.h"],
+    "pq_conv_tc_kernel": ["conv_tc.cuh", "pq_device.cuh", "pq_internal.h"],
+    "pq_conv_tc_kernel<FP4, quantise-on-load>": ["conv_tc.cuh", "pq_device.cuh", "pq_internal.h"],
 }
 
 

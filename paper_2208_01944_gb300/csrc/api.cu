@@ -142,6 +142,7 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
   // activation offset (the operand's tap t = position * R + slice)
   const int R = wslices_of(d);
   const int taps = d->kh * d->kw * R;
+  p.ipt = 1;
   const int qa = (1 << d->bits_a) - 1;
   const int qw = 1 << (d->bits_w - 1);
   // Coverage of the tensor-core kernel.
@@ -172,7 +173,6 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
   p.N = d->N;
   p.Ho = Ho;
   p.Wo = Wo;
-  p.P_out = static_cast<int64_t>(d->N) * Ho * Wo;
   p.G = d->G;
   p.Cin_g = d->Cin_g;
   p.Cout_g = d->Cout_g;
@@ -195,6 +195,7 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
   const int Wh = flat ? 0 : Wo + cmax - cmin;
   // Stride phases used by the taps, and each tap's (phase, offset).
   std::vector<Phase> phases;
+  int tap_phase[pq::kMaxTaps], tap_off[pq::kMaxTaps];  // stride phase and position offset of each tap in its plane
   int off_max = 0;
   if (!flat) {
     for (int i = 0; i < d->kh; ++i) {
@@ -209,17 +210,17 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
         }
         for (int r = 0; r < R; ++r) {
           const int t = (i * d->kw + j) * R + r;
-          p.tap_phase[t] = idx;
-          p.tap_off[t] = (floor_div(i - d->pad, s) - rmin) * Wh + (floor_div(j - d->pad, s) - cmin);
-          off_max = std::max(off_max, p.tap_off[t]);
+          tap_phase[t] = idx;
+          tap_off[t] = (floor_div(i - d->pad, s) - rmin) * Wh + (floor_div(j - d->pad, s) - cmin);
+          off_max = std::max(off_max, tap_off[t]);
         }
       }
     }
   } else {
     phases.push_back({0, 0});
     for (int r = 0; r < R; ++r) {
-      p.tap_phase[r] = 0;
-      p.tap_off[r] = 0;
+      tap_phase[r] = 0;
+      tap_off[r] = 0;
     }
   }
   p.nph = static_cast<int>(phases.size());
@@ -246,6 +247,10 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
   const double mma_acc_ns = static_cast<double>(p.taps) * (d->Cin_g / (32 * cpb)) * mma_ns;  // one accumulator
   // (quantise-on-load keeps the copy warps busy converting: two epilogue groups)
   const bool tma_operand = !quant_in && c16 && d->stride == 1 && (flat || Wh <= 128);
+  const bool multi_ok =
+      tma_operand && !p2 && !flat && d->pad < std::min(d->kh, d->kw) && d->H + d->pad <= 256;
+  // (32-bit offsets within the images of a tile)
+  const int64_t multi_bytes = static_cast<int64_t>(Ho) * Wo * d->G * d->Cout_g;
   const int epi_groups = tma_operand ? pq::kEpiGroups + 1 : pq::kEpiGroups;
   const int unit_cols = (f4 && p.Nblk % 32 == 0) ? 32 : 16;
   const int units_per_acc = p.Nblk / unit_cols;
@@ -253,7 +258,7 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
   const double w_unit_bytes = static_cast<double>(p.taps) * d->Cin_g * p.Nblk / cpb;
   const double w_stream_ns = w_unit_bytes > 160.0 * 1024.0 ? w_unit_bytes / 40.0 : 0.0;  // per item
   const int tmem_avail = f4 ? 512 - 32 : 512;  // FP4: 32 columns hold the scale factors
-  int best_mt = 0, best_ht = 0, best_tpi = 0, best_acc = 0;
+  int best_mt = 0, best_ht = 0, best_tpi = 0, best_acc = 0, best_ipt = 1;
   double best_cost = 0.0;
   for (int MT : {1, 2, 3, 4}) {
     // flat tiles: up to two accumulators (by TMA, one 128-position box each); the
@@ -261,7 +266,7 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
     if (flat && (MT > 2 || ((p2 || quant_in) && MT > 1))) continue;
     int acc_stages = (2 * MT * p.Npow2 <= tmem_avail) ? 2 : ((MT * p.Npow2 <= tmem_avail) ? 1 : 0);
     if (acc_stages == 0) continue;
-    int ht = 0, tpi = 0;
+    int ht = 0, tpi = 0, ipt = 1;
     if (flat) {
       tpi = static_cast<int>((static_cast<int64_t>(Ho) * Wo + MT * 128 - 1) / (MT * 128));
     } else {
@@ -269,6 +274,21 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
       if (ht_max < 1) continue;
       tpi = (Ho + ht_max - 1) / ht_max;
       ht = (Ho + tpi - 1) / tpi;
+      // Several whole images per tile where TMA loads the operand as it is and the
+      // accumulators hold more than one: the last one needs (Ho - 1) rows and Wo more
+      // positions.  A 3x3 layer of 128x7x7 images, 2 groups of 512 channels (FP4): two
+      // images per 128 rows instead of one, the streamed weights read half as often,
+      // 32.8 -> 22.5 us.
+      const int pos_img = (d->H + d->pad) * (d->W + d->pad);
+      const int last = (Ho - 1) * (d->W + d->pad) + Wo;
+      if (multi_ok && MT * 128 >= last && multi_bytes <= (1LL << 30) / 512)
+        ipt = std::min(std::min((MT * 128 - last) / pos_img + 1, d->N), 256);
+      if (ipt > 1) {
+        tpi = 1;
+        ht = Ho;
+      } else {
+        ipt = 1;
+      }
     }
     if (quant_in) {
       // two fp32 staging stages (128 bytes per position) and two operand stages
@@ -284,12 +304,13 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
     const int units = MT * units_per_acc;
     const double epi_ns = ((units + epi_groups - 1) / epi_groups) * unit_ns;
     const double mma_side = std::max(MT * mma_acc_ns, w_stream_ns);
-    const double cost = static_cast<double>(tpi) * (500.0 + std::max(mma_side, epi_ns));
+    const double cost = static_cast<double>(tpi) / ipt * (500.0 + std::max(mma_side, epi_ns));
     const bool better = best_mt == 0 || acc_stages > best_acc || (acc_stages == best_acc && cost < best_cost * 0.98);
     if (better) {
       best_mt = MT;
       best_ht = ht;
       best_tpi = tpi;
+      best_ipt = ipt;
       best_acc = acc_stages;
       best_cost = cost;
     }
@@ -312,12 +333,26 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
   } else {
     p.Ht = best_ht;
     p.tiles_per_img = best_tpi;
-    p.tiles = static_cast<int64_t>(d->N) * best_tpi;
+    p.tiles = static_cast<int64_t>((d->N + best_ipt - 1) / best_ipt) * best_tpi;
     p.Wh = Wh;
     p.Wd = Wh;
     p.Hd = p.Ht + rmax - rmin;
     p.h_off = rmin;
     p.w_coord = cmin;
+    if (best_ipt > 1) {
+      // rows share their side padding and images their upper and lower padding
+      p.ipt = best_ipt;
+      p.Wh = d->W + d->pad;
+      p.Wd = p.Wh;
+      p.Hd = d->H + d->pad;
+      p.img_pos = p.Hd * p.Wd;
+      p.img_magic = static_cast<uint32_t>(((1ull << 32) + p.img_pos - 1) / p.img_pos);
+      off_max = 0;
+      for (int t = 0; t < taps; ++t) {
+        tap_off[t] = (t / R / d->kw) * p.Wh + (t / R) % d->kw;
+        off_max = std::max(off_max, tap_off[t]);
+      }
+    }
     if (p.Wd > 256 || p.Hd > 256) {
       if (pub) *pub = plan;
       return PQ_EUNSUPPORTED;
@@ -344,6 +379,16 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
       *lbo = plane;
       return round_up(*phase_bytes, 1024);
     }
+    if (p.ipt > 1) {
+      // after the last chunk's last image: its lower and right padding (zeroed once),
+      // and whatever the accumulators' unused rows reach
+      const uint32_t plane = static_cast<uint32_t>(p.ipt * p.img_pos) * 16u;
+      *phase_bytes = static_cast<uint32_t>(nch) * plane;
+      *lbo = plane;
+      const uint64_t tail = static_cast<uint64_t>(nch) * plane + 16ull * (d->pad * p.Wh + d->pad);
+      return round_up(std::max<uint64_t>(tail, static_cast<uint64_t>(nch - 1) * plane + 16ull * (p.MT * 128 + off_max)),
+                      1024);
+    }
     const uint32_t plane = static_cast<uint32_t>(p.Hd) * p.Wd * 16u;
     *phase_bytes = round_up(static_cast<uint64_t>(nch) * plane, 128);
     *lbo = plane;
@@ -352,7 +397,6 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
     return round_up(std::max<uint64_t>(static_cast<uint64_t>(p.nph) * (*phase_bytes), overrun), 1024);
   };
   const uint32_t q_pitch = 80;
-  const uint32_t f_pitch = 128;
   // Staging for every warp that runs the epilogue: the copy warps join it only when
   // TMA loads the activation operand as it is (not unpacked, not quantised).
   const bool third_group =
@@ -441,7 +485,6 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
   p.H = d->H;
   p.W = d->W;
   p.stride = d->stride;
-  p.C_in_total = d->G * d->Cin_g;
   p.img_pix = d->H * d->W;
   p.codes_c16 = c16 ? 1 : 0;
   p.codes_p2 = p2 ? 1 : 0;
@@ -464,9 +507,10 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
                  : p2 ? static_cast<uint32_t>(p.nch) * pk_box_w * (flat ? 1 : p.Hd) * 4u
                  : split ? static_cast<uint32_t>(p.nch) * (2 * p.Hd) * (2 * p.Wd) * 16u
                  : flat ? static_cast<uint32_t>(p.nch) * p.flat_box * 16u
+                 : p.ipt > 1 ? static_cast<uint32_t>(p.nch) * p.ipt * p.img_pos * 16u
                         : static_cast<uint32_t>(p.nph) * p.nch * p.Hd * p.Wd * 16u;
   {
-    const int64_t C = p.C_in_total, H = d->H, W = d->W;
+    const int64_t C = static_cast<int64_t>(d->G) * d->Cin_g, H = d->H, W = d->W;
     if (c16) {
       // 16-byte chunks of 16 channels (32 for FP4 nibbles)
       p.ld_pix = 16;
@@ -486,9 +530,13 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
   p.lbo_a = lbo;
   p.a_phase_bytes = phase_bytes;
   for (int t = 0; t < taps; ++t)
-    p.tap_a16[t] = (static_cast<uint32_t>(p.tap_phase[t]) * phase_bytes + static_cast<uint32_t>(p.tap_off[t]) * 16u) >> 4;
+    p.tap_a16[t] = (static_cast<uint32_t>(tap_phase[t]) * phase_bytes + static_cast<uint32_t>(tap_off[t]) * 16u) >> 4;
   p.a_stage_bytes = stage_bytes;
   p.a_stages = a_stages;
+  if (p.ipt > 1) {
+    p.a_zero_off = phase_bytes;
+    p.a_zero_bytes = stage_bytes - phase_bytes;
+  }
   p.b_resident = resident ? 1 : 0;
   p.b_slice_bytes = static_cast<uint32_t>(KC) * p.Nblk / cpb;
   p.b_unit_bytes = static_cast<uint32_t>(unit_bytes);
@@ -507,13 +555,11 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
   p.smem_bar_off = p.smem_pk_off + static_cast<uint32_t>(a_stages) * p.pk_stage_bytes;
   p.smem_bytes = p.smem_bar_off + bar_bytes;
   p.stage_q_pitch = q_pitch;
-  p.stage_f_pitch = f_pitch;
   p.stage_warp_bytes = warp_stage;
   p.C_out_total = d->G * d->Cout_g;
   p.relu = d->relu;
   p.qmax_out = (1 << d->bits_out) - 1;
-  for (int g = 0; g < d->G; ++g) p.dst_group[g] = g;
-  for (int g = 0; g < d->G; ++g) p.src_group[g] = g;
+  for (int g = 0; g < d->G; ++g) p.group[g].dst = p.group[g].src = g;
 
   plan.supported = 1;
   plan.mode = p.mode;
@@ -685,6 +731,15 @@ bool encode_c16_map(const pq_layer_desc* d, const ConvParams& p, const void* q_d
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
   }
+  if (p.ipt > 1) {  // whole images: (row, image, chunk), so that a chunk's images are adjacent in the stage
+    cuuint64_t idims[4] = {2 * W, H, static_cast<cuuint64_t>(d->N), C16};
+    cuuint64_t istrides[3] = {W * 16, C16 * H * W * 16, H * W * 16};
+    cuuint32_t ibox[4] = {2u * static_cast<cuuint32_t>(p.Wd), static_cast<cuuint32_t>(p.Hd),
+                          static_cast<cuuint32_t>(p.ipt), static_cast<cuuint32_t>(p.nch)};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<void*>(q_dev), idims, istrides, ibox, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  }
   cuuint64_t dims[4] = {2 * W, H, C16, static_cast<cuuint64_t>(d->N)};
   cuuint64_t strides[3] = {W * 16, H * W * 16, C16 * H * W * 16};
   // stride 2 (a_split): the window of 2 Hd rows x 2 Wd positions
@@ -839,8 +894,8 @@ pq_status layer_fused_impl(const void* q_dev, const void* w_packed_dev, const pq
     if (u_in == nullptr || !valid_bounds(d->G, l_in, u_in)) return PQ_EINVAL;
     p.q_lu = 1;
     for (int g = 0; g < d->G; ++g) {
-      p.q_neg_l[g] = -l_in[g];
-      p.q_inv_r[g] = 1.0f / (u_in[g] - l_in[g]);
+      p.group[g].q_neg_l = -l_in[g];
+      p.group[g].q_mul = 1.0f / (u_in[g] - l_in[g]);
     }
     p.q_qp = static_cast<float>((1 << d->bits_a) - 1);
     p.q_qmax2 = static_cast<uint32_t>((1 << d->bits_a) - 1) * 0x00010001u;
@@ -851,7 +906,7 @@ pq_status layer_fused_impl(const void* q_dev, const void* w_packed_dev, const pq
       if (!std::isfinite(inv_s_in[g]) || !(inv_s_in[g] >= 0.0f) || (inv_s_in[g] != 0.0f && inv_s_in[g] < 1e-30f) ||
           inv_s_in[g] > 1e30f)
         return PQ_EINVAL;
-      p.q_inv_sat[g] = inv_s_in[g] * inv_two_b;
+      p.group[g].q_mul = inv_s_in[g] * inv_two_b;
     }
     p.q_two_b = static_cast<float>(1 << d->bits_a);
     p.q_qmax2 = static_cast<uint32_t>((1 << d->bits_a) - 1) * 0x00010001u;
@@ -863,13 +918,12 @@ pq_status layer_fused_impl(const void* q_dev, const void* w_packed_dev, const pq
   // that scaling and every product with an accumulator stay exact normal floats.
   auto usable = [](float m) { return std::isfinite(m) && (m == 0.0f || (std::fabs(m) > 1e-30f && std::fabs(m) < 1e30f)); };
   for (int g = 0; g < d->G; ++g) {
-    p.dst_group[g] = dst[g];
-    p.src_group[g] = src_group ? src_group[g] : g;
-    p.m_out[g] = m_out_host ? m_out_host[g] : 0.0f;
-    p.m_req[g] = m_req_host ? m_req_host[g] : 0.0f;
-    if (!usable(p.m_out[g]) || !usable(p.m_req[g])) return PQ_EINVAL;
-    p.m_out512[g] = p.m_out[g] * 512.0f;
-    p.m_req512[g] = p.m_req[g] * 512.0f;
+    p.group[g].dst = dst[g];
+    p.group[g].src = src_group ? src_group[g] : g;
+    const float m_out = m_out_host ? m_out_host[g] : 0.0f, m_req = m_req_host ? m_req_host[g] : 0.0f;
+    if (!usable(m_out) || !usable(m_req)) return PQ_EINVAL;
+    p.group[g].m_out512 = m_out * 512.0f;
+    p.group[g].m_req = m_req;
   }
   p.channel_shuffle = shuf.kind == 2 ? 1 : 0;
   // A per-channel scatter cannot write single 2-bit codes into packed bytes.
@@ -879,6 +933,8 @@ pq_status layer_fused_impl(const void* q_dev, const void* w_packed_dev, const pq
   p.acc_out = acc_out_dev;
   p.y_out = y_out_dev;
   p.q_out = static_cast<uint8_t*>(q_out_dev);
+  p.epi_general = shortcut_dev != nullptr || y_out_dev != nullptr || acc_out_dev != nullptr || p.channel_shuffle ||
+                  !p.codes_c16;
   p.err = pq::device_error_word();
   if (p.err == nullptr) return PQ_ECUDA;
   p.wait_limit_ns = g_wait_limit_ns.load();
@@ -890,7 +946,7 @@ pq_status layer_fused_impl(const void* q_dev, const void* w_packed_dev, const pq
   if (!quant_in && direct_out && q_out_dev != nullptr && shortcut_dev == nullptr && src_group == nullptr &&
       !p.channel_shuffle && plan_pointwise(d, &pw)) {
     for (int g = 0; g < d->G; ++g) {
-      pw.m_req15[g] = p.m_req[g] * (1.0f / 32768.0f);  // exact: m_req is 0 or above 1e-30 in magnitude
+      pw.m_req15[g] = p.group[g].m_req * (1.0f / 32768.0f);  // exact: m_req is 0 or above 1e-30 in magnitude
       pw.dst_group[g] = dst[g];
     }
     pw.w_packed = p.w_packed;

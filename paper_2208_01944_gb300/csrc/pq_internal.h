@@ -31,28 +31,52 @@ constexpr int kMaxSmem = 227 * 1024;
 
 enum ConvMode : int { kModeFlat = 0, kModeRows = 1 };
 
-// Everything the tensor-core conv kernel needs; filled by the host planner.
+// One group's scalars (source group g; src, q_mul and q_neg_l as the input side reads them).
+struct alignas(32) ConvGroup {
+  float m_out512;  // m_out * 2^9 (exact): applied to the raw accumulator, which holds acc * 2^-9
+  float m_req;     // as given: applied to the shortcut sum
+  float q_mul;     // quantise-on-load: fl(1/s) / 2^b, or with learned bounds fl(1 / fl(u - l))
+  float q_neg_l;   // learned bounds: -l
+  int dst, src;    // destination group; input group read by conv group g (identity, or the module's Eq. 8 permutation)
+};
+
+// Everything the tensor-core conv kernel needs; filled by the host planner.  The fields
+// that every role reads come first and the arrays last: a launch's parameters start cold
+// in the constant cache, a few hundred cycles a line.
 struct ConvParams {
   // ---- geometry
   int mode;               // kModeFlat or kModeRows
-  int N, Ho, Wo;          // output batch / spatial size
-  int64_t P_out;          // N * Ho * Wo
-  int G, Cin_g, Cout_g;
+  int Ho, Wo;             // output spatial size
+  int N, G, NB;           // images, groups, output-channel blocks per group
+  int Cin_g, Cout_g;
+  int tiles_per_img;      // rows mode
+  // Rows mode, several whole images per tile (ipt > 1; small images at stride 1): the
+  // stage holds, per 16-byte chunk, ipt images of img_rows = H + pad rows of Wh = W + pad
+  // positions, img_pos positions each.  An image's rows start with its left and upper
+  // padding; its right padding is the next row's left one and its lower padding the next
+  // image's upper one (after the last image, the next chunk's, and after the last chunk a
+  // zeroed tail), so 7x7 images take 64 accumulator rows instead of 81.
+  int ipt, img_pos;
+  uint32_t img_magic;     // ceil(2^32 / img_pos): m / img_pos = umulhi(m, img_magic) for small m
+  uint32_t wh_magic;      // ceil(2^32 / Wh) (rows mode): m / Wh = umulhi(m, wh_magic) for m < 2^24
   int Ht;                 // output rows per tile (rows mode)
   int Wh;                 // positions per tile row in the operand planes
-  int Hd, Wd;             // plane rows / columns loaded per phase
-  int h_off;              // first plane row = phase row oh0 + h_off
-  int w_coord;            // first plane column = phase column w_coord
-  int H, W, stride;       // input geometry
-  int C_in_total;         // G * Cin_g (bytes per input pixel)
+  int flat_box;           // pixels per flat-mode tile (= MT * 128)
   int img_pix;            // H * W (flat mode tiles stay inside one image)
-  int codes_c16;          // 1: input and output codes in the channel-blocked layout [N][C/16][H][W][16]
-  int codes_p2;           // 1: channel-blocked 2-bit codes packed four to a byte ([N][C/16][H][W][4 B])
-  // 1: 2-bit codes as packed FP4 (E2M1) nibbles, [N][C/32][H][W][16 B], read by the
-  // block-scaled FP4 MMA; one 16-byte chunk then holds 32 channels.
-  int codes_f4;
-  int chunk_shift;        // log2(channels per 16-byte chunk): 4, or 5 for FP4 codes
-  uint32_t sf_col;        // FP4: first TMEM column of the (uniform) block scale factors
+  int64_t tiles;          // tiles per (group, n-block) unit
+  int64_t items;          // tiles * G * NB
+  int64_t items_per_cta, items_rem;  // items / grid and items % grid: the first items_rem CTAs take one more
+  // pdl = 1: launched as a programmatic dependent of the previous kernel on the
+  // stream: a CTA's set-up (barriers, tensor memory) may run while that kernel's
+  // last CTAs still run; every global access waits for it to complete (stream
+  // order holds), and every CTA lets the next such launch start early.
+  int pdl;
+  // pdl_early_loads = 1 (the caller's PQ_LAYER_INPUTS_READY): only the epilogue
+  // warps (every global store) wait for the previous kernel; loads, quantisation
+  // and MMAs may start before it completes.
+  int pdl_early_loads;
+  // ---- pipeline
+  int a_tma;              // 1: warp 0 loads the A operand with one TMA per stage (channel-blocked codes, stride 1)
   // Packed activations come by TMA into a staging ring and the copy warps unpack
   // them into the operand stages (a_unpack = 1): staged rows of pk_box_w 32-bit
   // words starting pk_off words left of the tile's first position.
@@ -64,87 +88,72 @@ struct ConvParams {
   // Quantise-on-load (a_quant = 1): the input is fp32 NHWC; TMA stages boxes of 32
   // channels x all positions of a stage (128-byte rows, 128-byte swizzle) into the
   // staging ring and the copy warps quantise them into the operand stage:
-  // code = min(rint(sat(x * q_inv_sat[g]) * 2^b), Qp), q_inv_sat = fl(1/s) / 2^b.
-  int a_quant;
-  float q_inv_sat[kMaxG];
-  float q_two_b;
-  uint32_t q_qmax2;  // Qp in both 16-bit halves
-  // q_lu = 1: learned bounds l < u per group instead (Eq. 2 as trained):
-  // code = rint(sat((x - l) * q_inv_r[g]) * Qp), q_inv_r = fl(1 / fl(u - l)),
-  // q_neg_l = -l, q_qp = Qp; out-of-image positions are NaN-filled (code 0).
-  // pdl = 1: launched as a programmatic dependent of the previous kernel on the
-  // stream: a CTA's set-up (barriers, tensor memory) may run while that kernel's
-  // last CTAs still run; every global access waits for it to complete (stream
-  // order holds), and every CTA lets the next such launch start early.
-  int pdl;
-  // pdl_early_loads = 1 (the caller's PQ_LAYER_INPUTS_READY): only the epilogue
-  // warps (every global store) wait for the previous kernel; loads, quantisation
-  // and MMAs may start before it completes.
-  int pdl_early_loads;
-  int q_lu;
-  float q_neg_l[kMaxG];
-  float q_inv_r[kMaxG];
-  float q_qp;
-  uint32_t q_box_bytes;  // staging bytes per 32-channel box (a multiple of 1024: the 128B swizzle atom)
-  int pk_box_w, pk_off;
-  uint32_t pk_stage_bytes, smem_pk_off;
-  int a_tma;              // 1: warp 0 loads the A operand with one TMA per stage (channel-blocked codes, stride 1)
-  uint32_t a_tx_bytes;    // bytes one A stage receives (TMA mode)
-  // Activation copy addressing (cp.async mode), in bytes: code (n, ih, iw, c0 + 16 j) of the
-  // K block starting at channel c0 sits at n*ld_img + ih*ld_row + iw*ld_pix + ld_c0(c0) + j*ld_chunk,
-  // with ld_c0(c0) = c0 * ld_c0_mul / 16.
-  int64_t ld_img, ld_row, ld_pix, ld_chunk, ld_c0_mul;
-  int phase_a[kMaxPhases], phase_b[kMaxPhases];  // stride phase (row, column) of each plane set
-  uint32_t nch_magic;     // ceil(2^32 / nch): e / nch = umulhi(e, nch_magic) for small e
-  uint32_t wh_magic;      // ceil(2^32 / Wh) (rows mode): m / Wh = umulhi(m, wh_magic) for m < 2^24
-  int tiles_per_img;      // rows mode
-  int64_t tiles;          // tiles per (group, n-block) unit
-  int64_t items;          // tiles * G * NB
-  int64_t items_per_cta, items_rem;  // items / grid and items % grid: the first items_rem CTAs take one more
-  int NB, Nblk, Npow2;    // output-channel blocks, MMA N, TMEM column stride per accumulator
+  // code = min(rint(sat(x * q_mul) * 2^b), Qp), q_mul = fl(1/s) / 2^b; or with learned
+  // bounds l < u per group (q_lu = 1, Eq. 2 as trained)
+  // code = rint(sat((x - l) * q_mul) * Qp), q_mul = fl(1 / fl(u - l)), out-of-image
+  // positions NaN-filled (code 0).
+  int a_quant, q_lu;
+  int a_stages, b_stages; // operand ring; weight ring when streamed
+  int b_resident;         // 1: the whole unit's weights stay in shared memory
+  int acc_stages;         // TMEM accumulator buffers (ring of 1..kMaxAccStages)
+  int mma_warps;          // 2: two MMA warps take the items in turn (see mma_role)
+  int Nblk, Npow2;        // MMA N, TMEM column stride per accumulator
   int MT;                 // 128-row accumulators per tile
   int KC, n_kb, nch;      // channels per K block, K blocks, 16-byte chunks per K block
   int taps, nph;          // kh*kw, stride phases
-  int flat_box;           // pixels per flat-mode tile (= MT * 128)
-  int tap_phase[kMaxTaps];
-  int tap_off[kMaxTaps];  // position offset of each tap in the plane
-  uint32_t tap_a16[kMaxTaps];  // stage-relative start of each tap's A operand, in 16-byte units
+  int w_coord, h_off;     // first plane column = phase column w_coord, first row = phase row oh0 + h_off
+  int chunk_shift;        // log2(channels per 16-byte chunk): 4, or 5 for FP4 codes
   uint32_t lbo_a;         // byte stride between 16-byte K chunks of the A planes
+  uint32_t lbo_b;         // Nblk * 16
   uint32_t a_mt16;        // 16-byte units between the A operands of consecutive accumulators:
                           // 128 (one plane of positions), or nch * 128 (flat TMA: a box region each)
   uint32_t a_phase_bytes, a_stage_bytes;
-  int a_stages;
-  int b_resident;         // 1: the whole unit's weights stay in shared memory
+  uint32_t a_tx_bytes;    // bytes one A stage receives (TMA mode)
+  uint32_t a_zero_off, a_zero_bytes;  // zeroed tail of each operand stage (0 bytes: none)
   uint32_t b_slice_bytes; // one (K block, tap) slice: KC * Nblk bytes
   uint32_t b_unit_bytes;  // taps * Cin_g * Nblk
-  uint32_t lbo_b;         // Nblk * 16
-  int b_stages;           // ring stages when streamed
-  int acc_stages;         // TMEM accumulator buffers (ring of 1..kMaxAccStages)
-  int mma_warps;          // 2: two MMA warps take the items in turn (see mma_role)
+  uint32_t pk_stage_bytes;
+  uint32_t q_box_bytes;   // staging bytes per 32-channel box (a multiple of 1024: the 128B swizzle atom)
   uint32_t tmem_cols;
-  uint32_t smem_b_off, smem_stage_off, smem_bar_off, smem_bytes;
-  uint32_t stage_q_pitch, stage_f_pitch, stage_warp_bytes;
-  // ---- operands
-  const uint8_t* q_in;    // activation codes, NHWC
+  uint32_t sf_col;        // FP4: first TMEM column of the (uniform) block scale factors
+  uint32_t smem_b_off, smem_stage_off, smem_bar_off, smem_pk_off, smem_bytes;
   const uint8_t* w_packed;
   // ---- epilogue
-  int C_out_total;        // G * Cout_g
-  float m_out[kMaxG];     // as given: y = (float)acc * m_out
-  float m_req[kMaxG];     // as given: applied to the shortcut sum
-  float m_out512[kMaxG];  // m_out * 2^9 (exact): applied to the raw accumulator, which holds acc * 2^-9
-  float m_req512[kMaxG];  // m_req * 2^9 (exact)
-  int dst_group[kMaxG];
-  int src_group[kMaxG];  // input group read by conv group g (identity, or the module's Eq. 8 permutation)
-  int channel_shuffle;    // 1: destination channel co*G + g (per-channel scatter)
-  int relu;
-  int qmax_out;
+  int epi_general;        // int32 or fp32 outputs, a shortcut, NHWC codes or a channel shuffle; else
+                          // channel-blocked codes only, stored from registers
   const float* shortcut;
   int32_t* acc_out;
   float* y_out;
   uint8_t* q_out;
+  int C_out_total;        // G * Cout_g
+  int channel_shuffle;    // 1: destination channel co*G + g (per-channel scatter)
+  int relu;
+  int qmax_out;
+  int codes_c16;          // 1: input and output codes in the channel-blocked layout [N][C/16][H][W][16]
+  int codes_p2;           // 1: channel-blocked 2-bit codes packed four to a byte ([N][C/16][H][W][4 B])
+  // 1: 2-bit codes as packed FP4 (E2M1) nibbles, [N][C/32][H][W][16 B], read by the
+  // block-scaled FP4 MMA; one 16-byte chunk then holds 32 channels.
+  int codes_f4;
+  uint32_t stage_q_pitch, stage_warp_bytes;
   // ---- failure detection
   unsigned int* err;
   uint64_t wait_limit_ns;
+  // ---- the copy warps
+  int Hd, Wd;             // plane rows / columns loaded per phase
+  int H, W, stride;       // input geometry
+  int pk_box_w, pk_off;
+  float q_two_b;          // 2^b
+  uint32_t q_qmax2;       // Qp in both 16-bit halves
+  float q_qp;             // Qp
+  uint32_t nch_magic;     // ceil(2^32 / nch): e / nch = umulhi(e, nch_magic) for small e
+  // Activation copy addressing (cp.async mode), in bytes: code (n, ih, iw, c0 + 16 j) of the
+  // K block starting at channel c0 sits at n*ld_img + ih*ld_row + iw*ld_pix + ld_c0(c0) + j*ld_chunk,
+  // with ld_c0(c0) = c0 * ld_c0_mul / 16.
+  const uint8_t* q_in;    // activation codes, NHWC
+  int64_t ld_img, ld_row, ld_pix, ld_chunk, ld_c0_mul;
+  int phase_a[kMaxPhases], phase_b[kMaxPhases];  // stride phase (row, column) of each plane set
+  ConvGroup group[kMaxG];
+  uint32_t tap_a16[kMaxTaps];  // stage-relative start of each tap's A operand, in 16-byte units
 };
 
 // The pointwise kernel (1x1, stride 1, pad 0 layers, channel-blocked codes in

@@ -846,3 +846,47 @@ def test_quantize_layer_fused_special_inputs(B):
     a_ref, y_ref, q_ref = oracle.epilogue(acc, c.G, ref["m_out"], ref["m_req"], c.kind, c.shift, None, None, True, c.bo)
     ref2 = dict(ref, x=x, q=q, acc_ref=a_ref, y_ref=y_ref, q_ref=q_ref)
     assert_layer_parity(c, ref2, _run_quant_fused(B, c, ref2, 2))
+
+
+# ------------------------------------------------- tiles and units at their edges
+# Several whole images per tile: batches that the tile's image count does not divide,
+# images whose padding is shared by neighbours (pad 0, 1, 2), every epilogue.
+MULTI_CASES = [
+    Case(5, 7, 7, 2, 64, 64, 3, 1, 1, seed=201),
+    Case(9, 5, 6, 2, 128, 64, 3, 1, 1, shortcut=True, seed=202),
+    Case(7, 6, 4, 1, 64, 128, 5, 1, 2, kind=0, seed=203),
+    Case(11, 8, 7, 3, 64, 32, 3, 1, 0, kind=3, perm=(2, 0, 1), relu=False, seed=204),
+    Case(4, 1, 3, 2, 64, 64, 3, 1, 1, seed=205),
+    Case(2, 10, 10, 2, 64, 64, 3, 1, 1, shortcut=True, relu=False, seed=206),
+]
+
+
+@pytest.mark.parametrize("fmt", [2, 4], ids=["c16", "fp4"])
+@pytest.mark.parametrize("c", MULTI_CASES, ids=str)
+def test_tiles_of_several_images_match_oracle(B, c, fmt):
+    d = B.layer_desc(c.N, c.H, c.W, c.G, c.Cin, c.Cout, c.k, c.stride, c.pad, code_format=fmt)
+    assert B.palquant_conv_plan(d).tiles < c.N, "the tile holds one image only"
+    ref = prepare(c)
+    assert_layer_parity(c, ref, run_gpu(c, ref, fmt=fmt))
+    if not c.shortcut:
+        assert_layer_parity(c, ref, run_gpu(c, ref, outputs=("q",), fmt=fmt))
+
+
+def test_tiles_of_several_images_channel_shuffle_matches_oracle(B):
+    c = Case(5, 7, 7, 2, 64, 64, 3, 1, 1, kind=2, seed=207)
+    ref = prepare(c)
+    assert_layer_parity(c, ref, run_gpu(c, ref, fmt=2))
+
+
+# Units of a single tile: a CTA's items change their weights every time, so that each of
+# the two MMA warps sees units of which it has no item.
+@pytest.mark.parametrize("c,fmt", [(Case(1, 5, 5, 64, 64, 384, 3, 1, 1, seed=211), 4),
+                                   (Case(1, 4, 6, 64, 32, 272, 3, 1, 1, seed=212), 2),
+                                   (Case(1, 3, 3, 64, 32, 1040, 1, 1, 0, seed=213), 2)], ids=str)
+def test_units_of_one_tile_match_oracle(B, c, fmt):
+    d = B.layer_desc(c.N, c.H, c.W, c.G, c.Cin, c.Cout, c.k, c.stride, c.pad, code_format=fmt)
+    p = B.palquant_conv_plan(d)
+    assert p.tiles == 1 and p.work_items > 152 and p.weights_resident == 1
+    ref = prepare(c)
+    assert_layer_parity(c, ref, run_gpu(c, ref, fmt=fmt))
+    assert_layer_parity(c, ref, run_gpu(c, ref, outputs=("q",), fmt=fmt))
