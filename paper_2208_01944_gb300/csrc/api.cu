@@ -123,8 +123,21 @@ struct Phase {
 // (no int32 or fp32 outputs), which the epilogue stores straight from registers,
 // so the plan reserves no per-warp staging for it.  shortcut: the call reads a
 // shortcut (two staging buffers per warp).
+// tile: the tile to plan with (chosen here when NULL).
+struct Tile {
+  int MT = 0;            // accumulators per tile
+  int ht = 0, tpi = 0;   // rows per tile, tiles per image (rows mode)
+  int ipt = 1;           // images per tile
+  int acc_stages = 0;
+  int nsub = 1;          // parts that a block of output channels is split into
+  double cost = 0.0;
+};
+
+constexpr int kPlanSMs = 152;  // SMs the planner counts on
+
 pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, std::vector<Phase>* phases_out,
-                    bool quant_in = false, bool direct_out = false, bool shortcut = false) {
+                    bool quant_in = false, bool direct_out = false, bool shortcut = false,
+                    const Tile* tile = nullptr) {
   // Epilogue staging per warp: 32 rows of up to 32 fp32/int32 values (128 bytes,
   // chunk-swizzled), twice with a shortcut (the next unit's rows are fetched into
   // the second buffer), or 32 rows of 16 code bytes at a pitch of 80 bytes (an odd
@@ -143,6 +156,7 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
   const int R = wslices_of(d);
   const int taps = d->kh * d->kw * R;
   p.ipt = 1;
+  p.nsub = 1;
   const int qa = (1 << d->bits_a) - 1;
   const int qw = 1 << (d->bits_w - 1);
   // Coverage of the tensor-core kernel.
@@ -258,22 +272,24 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
   const double w_unit_bytes = static_cast<double>(p.taps) * d->Cin_g * p.Nblk / cpb;
   const double w_stream_ns = w_unit_bytes > 160.0 * 1024.0 ? w_unit_bytes / 40.0 : 0.0;  // per item
   const int tmem_avail = f4 ? 512 - 32 : 512;  // FP4: 32 columns hold the scale factors
-  int best_mt = 0, best_ht = 0, best_tpi = 0, best_acc = 0, best_ipt = 1;
-  double best_cost = 0.0;
-  for (int MT : {1, 2, 3, 4}) {
+  // The tile of MT accumulators of n_cols columns; false where it does not fit.
+  auto tile_of = [&](int MT, int n_cols, Tile* t) -> bool {
     // flat tiles: up to two accumulators (by TMA, one 128-position box each); the
     // packed 2-bit path stages one box
-    if (flat && (MT > 2 || ((p2 || quant_in) && MT > 1))) continue;
-    int acc_stages = (2 * MT * p.Npow2 <= tmem_avail) ? 2 : ((MT * p.Npow2 <= tmem_avail) ? 1 : 0);
-    if (acc_stages == 0) continue;
-    int ht = 0, tpi = 0, ipt = 1;
+    if (flat && (MT > 2 || ((p2 || quant_in) && MT > 1))) return false;
+    const int npow2 = next_pow2(n_cols);
+    t->MT = MT;
+    t->acc_stages = (2 * MT * npow2 <= tmem_avail) ? 2 : ((MT * npow2 <= tmem_avail) ? 1 : 0);
+    if (t->acc_stages == 0) return false;
+    t->ht = 0;
+    t->ipt = 1;
     if (flat) {
-      tpi = static_cast<int>((static_cast<int64_t>(Ho) * Wo + MT * 128 - 1) / (MT * 128));
+      t->tpi = static_cast<int>((static_cast<int64_t>(Ho) * Wo + MT * 128 - 1) / (MT * 128));
     } else {
       const int ht_max = (MT * 128) / Wh;
-      if (ht_max < 1) continue;
-      tpi = (Ho + ht_max - 1) / ht_max;
-      ht = (Ho + tpi - 1) / tpi;
+      if (ht_max < 1) return false;
+      t->tpi = (Ho + ht_max - 1) / ht_max;
+      t->ht = (Ho + t->tpi - 1) / t->tpi;
       // Several whole images per tile where TMA loads the operand as it is and the
       // accumulators hold more than one: the last one needs (Ho - 1) rows and Wo more
       // positions.  A 3x3 layer of 128x7x7 images, 2 groups of 512 channels (FP4): two
@@ -282,45 +298,102 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
       const int pos_img = (d->H + d->pad) * (d->W + d->pad);
       const int last = (Ho - 1) * (d->W + d->pad) + Wo;
       if (multi_ok && MT * 128 >= last && multi_bytes <= (1LL << 30) / 512)
-        ipt = std::min(std::min((MT * 128 - last) / pos_img + 1, d->N), 256);
-      if (ipt > 1) {
-        tpi = 1;
-        ht = Ho;
+        t->ipt = std::min(std::min((MT * 128 - last) / pos_img + 1, d->N), 256);
+      if (t->ipt > 1) {
+        t->tpi = 1;
+        t->ht = Ho;
       } else {
-        ipt = 1;
+        t->ipt = 1;
       }
     }
     if (quant_in) {
       // two fp32 staging stages (128 bytes per position) and two operand stages
       // (32 bytes per position) must fit beside the weights (resident, or a
       // two-slice ring) and the epilogue staging
-      const uint64_t npos = flat ? 128u : static_cast<uint64_t>(ht + rmax - rmin) * Wh;
-      const uint64_t w_unit = static_cast<uint64_t>(taps) * d->Cin_g * p.Nblk / cpb;
-      const uint64_t w_min = 2ull * round_up(32ull * p.Nblk, 1024);  // a streamed ring at least (resident when it fits)
+      const uint64_t npos = flat ? 128u : static_cast<uint64_t>(t->ht + rmax - rmin) * Wh;
+      const uint64_t w_min = 2ull * round_up(32ull * n_cols, 1024);  // a streamed ring at least (resident when it fits)
       const uint64_t need = 2ull * (cpb * round_up(npos * 128, 1024) + round_up(npos * 32, 1024)) + w_min +
                             static_cast<uint64_t>(pq::kEpiWarps) * warp_stage + 1024;
-      if (need > pq::kMaxSmem - 1024) continue;
+      if (need > pq::kMaxSmem - 1024) return false;
     }
-    const int units = MT * units_per_acc;
-    const double epi_ns = ((units + epi_groups - 1) / epi_groups) * unit_ns;
-    const double mma_side = std::max(MT * mma_acc_ns, w_stream_ns);
-    const double cost = static_cast<double>(tpi) / ipt * (500.0 + std::max(mma_side, epi_ns));
-    const bool better = best_mt == 0 || acc_stages > best_acc || (acc_stages == best_acc && cost < best_cost * 0.98);
-    if (better) {
-      best_mt = MT;
-      best_ht = ht;
-      best_tpi = tpi;
-      best_ipt = ipt;
-      best_acc = acc_stages;
-      best_cost = cost;
+    return true;
+  };
+  auto items_of = [&](const Tile& t) -> int64_t {
+    return static_cast<int64_t>((d->N + t.ipt - 1) / t.ipt) * t.tpi * d->G * p.NB * t.nsub;
+  };
+  Tile best;
+  if (tile != nullptr) {
+    best = *tile;
+  } else {
+    for (int MT : {1, 2, 3, 4}) {
+      Tile t;
+      if (!tile_of(MT, p.Nblk, &t)) continue;
+      const int units = MT * units_per_acc;
+      const double epi_ns = ((units + epi_groups - 1) / epi_groups) * unit_ns;
+      const double mma_side = std::max(MT * mma_acc_ns, w_stream_ns);
+      t.cost = static_cast<double>(t.tpi) / t.ipt * (500.0 + std::max(mma_side, epi_ns));
+      if (best.MT == 0 || t.acc_stages > best.acc_stages ||
+          (t.acc_stages == best.acc_stages && t.cost < best.cost * 0.98))
+        best = t;
+    }
+    if (best.MT == 0) {
+      if (pub) *pub = plan;
+      return PQ_EUNSUPPORTED;
+    }
+    // Few items for the chip: the longest CTA's time counts, in whole items, and a block
+    // of output channels may be split between CTAs (each loads its columns of the packed
+    // weights).  Each item costs as above, with the general epilogue's units at 1500 ns
+    // (32 columns) or 850; the weights that stay are loaded once, streamed ones for every
+    // item, at 80 B/ns; the shorter of the MMAs and the epilogue is paid once more.  The
+    // network at batch 1 (8 to 20 items a layer before): 218 -> 197 us.  A layer that the
+    // rule above cannot plan stays refused, and keeps that plan where this one has none.
+    if (items_of(best) < 8 * kPlanSMs && d->N > 0) {
+      Tile fast;
+      const int64_t items0 = items_of(best);
+      for (int nsub : {1, 2, 4, 8}) {
+        const int n_cols = p.Nblk / nsub;
+        if (nsub > 1 && (items0 >= kPlanSMs || p.Nblk % (32 * nsub) != 0)) continue;
+        for (int MT : {1, 2, 3, 4}) {
+          Tile t;
+          t.nsub = nsub;
+          if (!tile_of(MT, n_cols, &t)) continue;
+          const bool wide = direct_out ? f4 && n_cols % 32 == 0 : n_cols % 32 == 0;  // 32-column units
+          const int units = MT * n_cols / (wide ? 32 : 16);
+          const double u_ns = direct_out ? (wide ? 550.0 : 430.0) : (wide ? 1500.0 : 850.0);
+          const double epi = ((units + epi_groups - 1) / epi_groups) * u_ns;
+          const int np2 = next_pow2(n_cols);
+          const double w_bytes = static_cast<double>(taps) * d->Cin_g * n_cols / cpb;
+          const bool stream = w_bytes > 160.0 * 1024.0;
+          const double mma = std::max(static_cast<double>(MT) * taps * (d->Cin_g / (32 * cpb)) *
+                                          std::max(32.0 + np2 / 4.0, np2 / 2.0) * ns_per_clk,
+                                      stream ? w_bytes / 80.0 : 0.0);
+          const int64_t waves = (items_of(t) + kPlanSMs - 1) / kPlanSMs;
+          const double item_ns = 500.0 + (t.acc_stages == 1 && waves > 1 ? mma + epi : std::max(mma, epi));
+          t.cost = (stream ? 0.0 : w_bytes / 80.0) + waves * item_ns + std::min(mma, epi);
+          if (fast.MT == 0 || t.cost < fast.cost * 0.97) fast = t;
+        }
+      }
+      const bool differs = fast.MT != 0 && (fast.MT != best.MT || fast.nsub != 1);
+      if (differs) {
+        pq_status base = plan_conv(d, P, pub, phases_out, quant_in, direct_out, shortcut, &best);
+        if (base != PQ_OK) return base;
+        ConvParams pf;
+        pq_conv_plan pubf;
+        if (plan_conv(d, &pf, &pubf, nullptr, quant_in, direct_out, shortcut, &fast) == PQ_OK) {
+          if (P) *P = pf;
+          if (pub) *pub = pubf;
+        }
+        return PQ_OK;
+      }
     }
   }
-  if (best_mt == 0) {
-    if (pub) *pub = plan;
-    return PQ_EUNSUPPORTED;
-  }
-  p.MT = best_mt;
-  p.acc_stages = best_acc;
+  const int best_ht = best.ht, best_tpi = best.tpi, best_ipt = best.ipt;
+  p.nsub = best.nsub;
+  p.NB *= best.nsub;
+  p.Nblk /= best.nsub;
+  p.Npow2 = next_pow2(p.Nblk);
+  p.MT = best.MT;
+  p.acc_stages = best.acc_stages;
   if (flat) {
     // Flat tiles are runs of flat_box pixels inside one image.
     p.flat_box = p.MT * 128;
@@ -362,7 +435,7 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
       p.phase_b[i] = phases[i].b;
     }
   }
-  p.items = p.tiles * d->G * NB;
+  p.items = p.tiles * d->G * p.NB;
   // K blocks, weights residency and pipeline depth under the shared-memory budget.
   const uint32_t budget = pq::kMaxSmem - 1024;
   auto a_stage_bytes = [&](int KC, uint32_t* phase_bytes, uint32_t* lbo) -> uint32_t {
@@ -782,6 +855,24 @@ bool encode_f32_map(const pq_layer_desc* d, const ConvParams& p, const void* x_d
              fill) == CUDA_SUCCESS;
 }
 
+// Tensor map of the packed weights for a plan that splits the blocks of output
+// channels: rows of one 16-byte chunk of every channel of a block (8-byte elements),
+// boxes of a K block's chunks x the part's channels.
+bool encode_weight_map(const pq_layer_desc* d, const ConvParams& p, CUtensorMap* map) {
+  EncodeTiledFn enc = encode_fn();
+  if (enc == nullptr) return false;
+  std::memset(map, 0, sizeof(*map));
+  const uint64_t row = static_cast<uint64_t>(p.Nblk) * p.nsub * 16;  // bytes of a chunk's row
+  const uint64_t bytes = static_cast<uint64_t>(d->G) * d->Cout_g * p.taps * d->Cin_g / (p.codes_f4 ? 2 : 1);
+  cuuint64_t dims[2] = {row / 8, bytes / row};
+  cuuint64_t strides[1] = {row};
+  cuuint32_t box[2] = {2u * static_cast<cuuint32_t>(p.Nblk), static_cast<cuuint32_t>(p.nch)};
+  cuuint32_t es[2] = {1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<uint8_t*>(p.w_packed), dims, strides, box, es,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 bool encode_pw_map(const pq_layer_desc* d, const pq::PwParams& p, const void* q_dev, CUtensorMap* map) {
   EncodeTiledFn enc = encode_fn();
   if (enc == nullptr) return false;
@@ -811,17 +902,19 @@ bool encode_pw_map(const pq_layer_desc* d, const pq::PwParams& p, const void* q_
 template <typename F>
 void for_each_packed(const ConvParams& p, int kw, F&& f) {
   const int E = 16 << (p.chunk_shift - 4);
+  // the packing's blocks: whole ones, however the plan splits them between CTAs
+  const int NB = p.NB / p.nsub, Nblk = p.Nblk * p.nsub;
   for (int g = 0; g < p.G; ++g)
-    for (int nb = 0; nb < p.NB; ++nb)
+    for (int nb = 0; nb < NB; ++nb)
       for (int kb = 0; kb < p.n_kb; ++kb)
         for (int t = 0; t < p.taps; ++t)
           for (int j = 0; j < p.nch; ++j)
-            for (int c = 0; c < p.Nblk; ++c)
+            for (int c = 0; c < Nblk; ++c)
               for (int e = 0; e < E; ++e) {
-                const int u = g * p.NB + nb;
+                const int u = g * NB + nb;
                 const size_t dst =
-                    ((((static_cast<size_t>(u) * p.taps + t) * p.n_kb + kb) * p.nch + j) * p.Nblk + c) * E + e;
-                const int co = nb * p.Nblk + c;
+                    ((((static_cast<size_t>(u) * p.taps + t) * p.n_kb + kb) * p.nch + j) * Nblk + c) * E + e;
+                const int co = nb * Nblk + c;
                 const int ci = kb * p.KC + j * E + e;
                 const int i = t / kw, jj = t % kw;
                 const size_t src = (((static_cast<size_t>(g) * p.Cout_g + co) * (p.taps / kw) + i) * kw + jj) * p.Cin_g + ci;
@@ -975,7 +1068,10 @@ pq_status layer_fused_impl(const void* q_dev, const void* w_packed_dev, const pq
   } else if (p.a_tma && !encode_c16_map(d, p, q_dev, &map)) {
     return PQ_ECUDA;
   }
-  if (pq::launch_conv_tc(p, map, grid, static_cast<cudaStream_t>(stream)) != 0) return PQ_ECUDA;
+  CUtensorMap w_map;
+  std::memset(&w_map, 0, sizeof(w_map));
+  if (p.nsub > 1 && !encode_weight_map(d, p, &w_map)) return PQ_ECUDA;
+  if (pq::launch_conv_tc(p, map, w_map, grid, static_cast<cudaStream_t>(stream)) != 0) return PQ_ECUDA;
   return PQ_OK;
 }
 

@@ -9,7 +9,8 @@ namespace pq {
 const void* conv_kernel_f8(bool lu);
 const void* conv_kernel_f4(bool lu);
 
-int launch_conv_tc(const ConvParams& p, const CUtensorMap& tma_a, int grid, cudaStream_t stream) {
+int launch_conv_tc(const ConvParams& p, const CUtensorMap& tma_a, const CUtensorMap& tma_w, int grid,
+                   cudaStream_t stream) {
   // the attribute is set once per instance and device
   static int attr_set_for_device[4][64] = {{0}};
   int dev = 0;
@@ -32,7 +33,7 @@ int launch_conv_tc(const ConvParams& p, const CUtensorMap& tma_a, int grid, cuda
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = p.pdl ? 1 : 0;
-  void* args[] = {const_cast<ConvParams*>(&p), const_cast<CUtensorMap*>(&tma_a)};
+  void* args[] = {const_cast<ConvParams*>(&p), const_cast<CUtensorMap*>(&tma_a), const_cast<CUtensorMap*>(&tma_w)};
   const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

@@ -159,7 +159,8 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, const W
 // activation operand of each stage as one TMA load (every plane row is a
 // contiguous run there).
 // --------------------------------------------------------------------------
-__device__ __forceinline__ void producer_role(const ConvParams& p, const CUtensorMap* tmA, const Bars& bars,
+__device__ __forceinline__ void producer_role(const ConvParams& p, const CUtensorMap* tmA, const CUtensorMap* tmW,
+                                              const Bars& bars,
                                               uint32_t a_base, uint32_t b_base, uint32_t pk_base, int64_t it0,
                                               int64_t it1, const WaitCtx& ctx) {
   Ring ra{0, 0, static_cast<uint32_t>(p.a_stages)};
@@ -225,6 +226,12 @@ __device__ __forceinline__ void producer_role(const ConvParams& p, const CUtenso
       item_next(p, a_item);
     }
   };
+  // Slice k = tap * n_kb + (K block) of a unit that is a part of a packed block: the
+  // part's channels of every chunk.  x counts 8-byte elements, two per channel.
+  auto load_w = [&](int unit, int k, uint32_t dst, uint32_t bar) {
+    const int blk = unit / p.nsub, sub = unit - blk * p.nsub;
+    tma_load_2d(dst, tmW, sub * 2 * p.Nblk, (blk * p.taps * p.n_kb + k) * p.nch, bar);
+  };
   if (p.b_resident) {
     for (int64_t it = it0; it < it1 && ok; ++it, item_next(p, item)) {
       const int64_t unit = item.unit;
@@ -232,9 +239,14 @@ __device__ __forceinline__ void producer_role(const ConvParams& p, const CUtenso
         if (!mbar_wait(bars.b_empty(rb.stage), rb.phase ^ 1u, ctx)) break;
         const uint32_t bar = bars.b_full(rb.stage);
         mbar_arrive_expect_tx(bar, p.b_unit_bytes);
-        const uint8_t* src = p.w_packed + static_cast<size_t>(unit) * p.b_unit_bytes;
-        for (uint32_t off = 0; off < p.b_unit_bytes; off += 65536u)
-          bulk_load(b_base + off, src + off, min(65536u, p.b_unit_bytes - off), bar);
+        if (p.nsub > 1) {
+          for (int k = 0; k < p.taps * p.n_kb; ++k)
+            load_w(item.unit, k, b_base + static_cast<uint32_t>(k) * p.b_slice_bytes, bar);
+        } else {
+          const uint8_t* src = p.w_packed + static_cast<size_t>(unit) * p.b_unit_bytes;
+          for (uint32_t off = 0; off < p.b_unit_bytes; off += 65536u)
+            bulk_load(b_base + off, src + off, min(65536u, p.b_unit_bytes - off), bar);
+        }
         rb.advance();
         ++b_issued;
         cur_unit = unit;
@@ -262,8 +274,13 @@ __device__ __forceinline__ void producer_role(const ConvParams& p, const CUtenso
           if (!mbar_wait(bars.b_empty(rb.stage), rb.phase ^ 1u, ctx)) { ok = false; break; }
           const uint32_t bar = bars.b_full(rb.stage);
           mbar_arrive_expect_tx(bar, p.b_slice_bytes);
-          const size_t slice = (static_cast<size_t>(unit) * p.taps + t) * p.n_kb + kb;  // tap-major packing
-          bulk_load(b_base + rb.stage * p.b_slice_bytes, p.w_packed + slice * p.b_slice_bytes, p.b_slice_bytes, bar);
+          const uint32_t dst = b_base + rb.stage * p.b_slice_bytes;
+          if (p.nsub > 1) {
+            load_w(item.unit, t * p.n_kb + kb, dst, bar);
+          } else {
+            const size_t slice = (static_cast<size_t>(unit) * p.taps + t) * p.n_kb + kb;  // tap-major packing
+            bulk_load(dst, p.w_packed + slice * p.b_slice_bytes, p.b_slice_bytes, bar);
+          }
           rb.advance();
           ++b_issued;
           if (a_left > 0 && a_issued <= block + 1 && mbar_test(a_slot(), ra.phase ^ 1u)) load_a();
@@ -1445,7 +1462,8 @@ __device__ __forceinline__ void epilogue_role(const ConvParams& p, const Bars& b
 // on the other's registers.
 template <bool F4, bool LU>
 __global__ void __launch_bounds__(kConvThreads, 1)
-    pq_conv_tc_kernel(const __grid_constant__ ConvParams p, const __grid_constant__ CUtensorMap tmA) {
+    pq_conv_tc_kernel(const __grid_constant__ ConvParams p, const __grid_constant__ CUtensorMap tmA,
+                      const __grid_constant__ CUtensorMap tmW) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -1526,7 +1544,8 @@ __global__ void __launch_bounds__(kConvThreads, 1)
   if (warp == 0) {
     if (lane == 0) {
       if (p.a_tma) prefetch_tmap(&tmA);
-      producer_role(p, &tmA, bars, a_base, b_base, base + p.smem_pk_off, it0, it1,
+      if (p.nsub > 1) prefetch_tmap(&tmW);
+      producer_role(p, &tmA, &tmW, bars, a_base, b_base, base + p.smem_pk_off, it0, it1,
                     WaitCtx{abort_flag, p.err, p.wait_limit_ns, PQ_ERR_PRODUCER});
     }
     __syncwarp();

@@ -98,6 +98,7 @@ struct ConvParams {
   int acc_stages;         // TMEM accumulator buffers (ring of 1..kMaxAccStages)
   int mma_warps;          // 2: two MMA warps take the items in turn (see mma_role)
   int Nblk, Npow2;        // MMA N, TMEM column stride per accumulator
+  int nsub;               // > 1: an output block is a part of the packing's (Nblk * nsub channels)
   int MT;                 // 128-row accumulators per tile
   int KC, n_kb, nch;      // channels per K block, K blocks, 16-byte chunks per K block
   int taps, nph;          // kh*kw, stride phases
@@ -192,7 +193,8 @@ struct PwParams {
 };
 
 // Host-side launch helpers implemented in the .cu files.
-int launch_conv_tc(const ConvParams& p, const CUtensorMap& tma_a, int grid, cudaStream_t stream);
+int launch_conv_tc(const ConvParams& p, const CUtensorMap& tma_a, const CUtensorMap& tma_w, int grid,
+                   cudaStream_t stream);
 int launch_pointwise_tc(const PwParams& p, const CUtensorMap& tma_a, int grid, cudaStream_t stream);
 int launch_bitsplit_act(const uint8_t* q, uint8_t* xs, int64_t N, int64_t HW, int C, int Ga, int B, int c16,
                         cudaStream_t stream);

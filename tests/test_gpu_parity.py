@@ -857,7 +857,7 @@ MULTI_CASES = [
     Case(7, 6, 4, 1, 64, 128, 5, 1, 2, kind=0, seed=203),
     Case(11, 8, 7, 3, 64, 32, 3, 1, 0, kind=3, perm=(2, 0, 1), relu=False, seed=204),
     Case(4, 1, 3, 2, 64, 64, 3, 1, 1, seed=205),
-    Case(2, 10, 10, 2, 64, 64, 3, 1, 1, shortcut=True, relu=False, seed=206),
+    Case(161, 10, 10, 2, 64, 64, 3, 1, 1, shortcut=True, relu=False, seed=206),
 ]
 
 
@@ -890,3 +890,24 @@ def test_units_of_one_tile_match_oracle(B, c, fmt):
     ref = prepare(c)
     assert_layer_parity(c, ref, run_gpu(c, ref, fmt=fmt))
     assert_layer_parity(c, ref, run_gpu(c, ref, outputs=("q",), fmt=fmt))
+
+
+# Few items for the chip: blocks of output channels split between CTAs, each loading its
+# columns of the packed weights (resident, and streamed slice by slice).
+SPLIT_CASES = [
+    (Case(1, 14, 14, 2, 256, 256, 3, 1, 1, seed=221), 4), (Case(1, 7, 9, 2, 512, 384, 3, 1, 1, shortcut=True, seed=222), 4),
+    (Case(1, 9, 9, 2, 64, 192, 3, 1, 1, seed=223), 2), (Case(1, 5, 4, 1, 1024, 256, 3, 1, 1, seed=224), 2),
+    (Case(1, 8, 8, 2, 64, 128, 3, 2, 1, relu=False, seed=225), 2), (Case(1, 6, 7, 3, 96, 256, 1, 1, 0, seed=226), 0),
+    (Case(2, 12, 12, 1, 128, 256, 1, 2, 0, kind=0, seed=227), 4),
+]
+
+
+@pytest.mark.parametrize("c,fmt", SPLIT_CASES, ids=str)
+def test_split_channel_blocks_match_oracle(B, c, fmt):
+    d = B.layer_desc(c.N, c.H, c.W, c.G, c.Cin, c.Cout, c.k, c.stride, c.pad, code_format=fmt)
+    many = B.layer_desc(4096, c.H, c.W, c.G, c.Cin, c.Cout, c.k, c.stride, c.pad, code_format=fmt)
+    assert B.palquant_conv_plan(d).n_blocks > B.palquant_conv_plan(many).n_blocks, "the blocks are not split"
+    ref = prepare(c)
+    assert_layer_parity(c, ref, run_gpu(c, ref, fmt=fmt))
+    if not c.shortcut:
+        assert_layer_parity(c, ref, run_gpu(c, ref, outputs=("q",), fmt=fmt))
