@@ -94,50 +94,56 @@ __global__ void __launch_bounds__(kF32Threads) pq_conv2d_f32_kernel(const float*
   }
 }
 
-// Two fp32 fused multiply-adds in one packed instruction: (d0, d1) = (a b0 + d0,
-// a b1 + d1), each with a single IEEE rounding like __fmaf_rn.
-__device__ __forceinline__ void fma2_rn(float& d0, float& d1, float a, float b0, float b1) {
-  asm("{\n.reg .b64 x, y, z;\nmov.b64 x, {%2, %2};\nmov.b64 y, {%3, %4};\nmov.b64 z, {%0, %1};\n"
-      "fma.rn.f32x2 z, x, y, z;\nmov.b64 {%0, %1}, z;\n}"
-      : "+f"(d0), "+f"(d1)
-      : "f"(a), "f"(b0), "f"(b1));
-}
-
 // The 7x7 stride-2 convolution of a 3-channel image to 128 channels (the
-// network's first layer).  One block of 256 threads per SM computes output
-// tiles of 16 rows x 16 columns; thread (row r, channel group g) holds the 16
-// pixels of tile row r and the 8 channels 8 g .. 8 g + 7: 128 sums, so that a
-// term costs four 16-byte input loads, two 16-byte weight loads and 64 packed
-// FMAs, with the registers to load the next term's operands while the current
-// one's FMAs run.  The input window of a tile (37 x 37 x 3 floats, zero outside
-// the image) is held split by column parity, channel-planar, in four copies
-// shifted by 0..3 positions: copy s of parity b holds at row i, position k the
-// window's column 2 (k + s) + b, so the 16 inputs of a thread for tap (kh, kw)
-// are positions 0..15, aligned, of copy kw / 2, parity kw % 2, row 2 r + kh.
-// The next tile's window comes into a plain copy in shared memory by cp.async
-// while the current one is computed, and is split into the copies between the
-// tile's two barriers.  The weights of a term are stored as two
-// halves of 4 channels per group ([147][2][16][4]): the 16 groups of a warp
-// read 256 contiguous bytes.  Per output the terms are added in (kh, kw, ci)
-// order like the generic kernel; the zero taps outside the image change
-// nothing: fma(0, w, acc) = acc for finite w, since a sum started at +0 is
-// never -0 under round-to-nearest.
+// network's first layer), bound by the FP32 FMAs (147 terms x 128 channels a pixel).
+//
+// A block of 256 threads per SM is two independent groups of four warps.  A group's
+// work item is a tile of 16 rows x PX columns and one half of the channels; its thread
+// (row r, channel group g) holds the PX pixels of row r and the 8 channels 8 g .. + 7
+// of the half, so a term costs four or five 16-byte input loads, two 16-byte weight
+// loads and 4 PX packed FMAs (PX = 16).  The groups run at their own pace, barriers
+// apart, and the second starts a part of a tile later: a group's other phases (input
+// split, pooling, stores, about a third of a tile's time when the whole block took them
+// together) then pass under the other group's FMAs.  128 images of 224x224 with the
+// pooling: 1204 us as one group of eight warps, 984 as two (30.7 T FMA/s; a probe of
+// the packed FMA alone sustains 36.1); one image 36 us, and 18 with 8-column tiles.
+//
+// The input window of a tile (37 rows x 2 PX + 5 columns x 3, zero outside the image)
+// lies split by column parity, channel-planar: parity b holds at row i, position k the
+// window's column 2 k + b, so the inputs of a thread for tap (kh, kw) are positions
+// kw / 2 .. of parity kw % 2, row 2 r + kh: whole 16-byte loads from position 0 on and
+// a compile-time choice of registers.  The next item's window comes into a plain copy
+// (the image's rows as they lie, in 16-byte pieces where their alignment allows) by
+// cp.async while the current one is computed, and is split between the item's two
+// barriers.  The weights of a term are stored as two halves of 4 channels per group
+// (rows of [2][16][4]): the 8 groups of a warp read 128 contiguous bytes.  Per output the
+// terms are added in (kh, kw, ci) order like the generic kernel; the zero taps outside
+// the image change nothing: fma(0, w, acc) = acc for finite w, since a sum started at
+// +0 is never -0 under round-to-nearest.
 constexpr int kStemK = 7, kStemS = 2, kStemP = 3, kStemCin = 3, kStemCout = 128;
-constexpr int kStemTH = 16, kStemTW = 16;
-constexpr int kStemThreads = 256;
+constexpr int kStemTH = 16;
+constexpr int kStemThreads = 256, kStemGroup = kStemThreads / 2;
+constexpr int kStemHalf = kStemCout / 2;                  // channels of an item
 constexpr int kStemIR = (kStemTH - 1) * kStemS + kStemK;  // 37 input rows
-constexpr int kStemIC = (kStemTW - 1) * kStemS + kStemK;  // 37 input columns
 constexpr int kStemTerms = kStemK * kStemK * kStemCin;    // 147
-constexpr int kStemRowF = 16;                             // positions per copy row
-constexpr int kStemPlaneF = kStemIR * kStemRowF;          // one (copy, parity, channel) plane
-constexpr int kStemCopyF = 2 * kStemCin * kStemPlaneF;    // one shifted copy
-constexpr int kStemXFloats = 4 * kStemCopyF;              // one window
-constexpr int kStemTileElems = kStemIR * kStemIC * kStemCin;                     // 4107
-constexpr int kStemLoads = (kStemTileElems + kStemThreads - 1) / kStemThreads;  // 17 per thread
-constexpr int kStemPoolRowF = 9 * kStemCout;  // a staged row of pooled columns (max pooling)
-constexpr int kStemRawF = (kStemTileElems + 3) / 4 * 4;  // the next window as it lies in the image
-constexpr size_t kStemSmem = (static_cast<size_t>(kStemTerms) * kStemCout + kStemXFloats + kStemRawF +
-                              (kStemTH / 2) * kStemPoolRowF) * sizeof(float);
+// floats between a term's weights: 128, and 4 more so that a warp that reads a channel's
+// terms in order (whole lines of the packed tensor) spreads them over the banks
+constexpr int kStemWF = kStemCout + 4;
+
+template <int PX>
+struct StemTile {
+  static constexpr int kIC = (PX - 1) * kStemS + kStemK;  // input columns
+  static constexpr int kRowF = PX + 4;                    // positions per plane row (16-byte multiple)
+  static constexpr int kPlaneF = kStemIR * kRowF;         // one (parity, channel) plane
+  static constexpr int kXF = 2 * kStemCin * kPlaneF;      // one window
+  static constexpr int kChunks = (3 + kIC * kStemCin + 3) / 4;  // 16-byte pieces of a window row, from 3 floats before it
+  static constexpr int kRawRowF = 4 * kChunks;
+  static constexpr int kRawF = kStemIR * kRawRowF;        // the next window as it lies in the image
+  static constexpr int kPC = PX / 2 + 1;                  // pooled columns that a tile touches
+  static constexpr int kPoolRowF = kPC * kStemHalf;       // a staged row of pooled columns
+  static constexpr int kGroupF = kXF + kRawF + (kStemTH / 2) * kPoolRowF;
+  static constexpr size_t kSmem = (static_cast<size_t>(kStemTerms) * kStemWF + 2 * kGroupF) * sizeof(float);
+};
 
 // Packed fp32 pairs in one 64-bit register (the low half first), and the packed
 // fused multiply-add on them: d = a b + d lane by lane, each lane with a single
@@ -154,128 +160,163 @@ __device__ __forceinline__ void ffma2(unsigned long long& d, unsigned long long 
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
 
-// One 4-byte asynchronous copy global -> shared, zero-filled when !valid.
+// One asynchronous copy of 4 or 16 bytes global -> shared, zero-filled when !valid.
 __device__ __forceinline__ void cp_async4(float* dst, const float* src, bool valid) {
   const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async16(float* dst, const float* src, bool valid) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(valid ? 16 : 0) : "memory");
 }
 
 // 3x3 stride-2 pad-1 max pooling of the stem tile held in registers (ReLU
 // outputs, so every value is >= 0, and pixels outside the output are 0).
 // Pooled row pr (0..8) of the tile covers stem rows 2 pr - 1 .. 2 pr + 1 and
-// pooled column pc (0..8) stem columns 2 pc - 1 .. 2 pc + 1 (tile-relative).
-// Columns: each thread reduces its row's 16 pixels to the 9 windows it sees.
-// Rows: the odd rows go through shared memory (`stage`) to the even rows'
-// threads, which complete pooled rows 1..7.  Windows that reach into a
-// neighbouring tile (pooled row 0 and 8, pooled column 0 and 8) are combined
-// across tiles by an integer atomic maximum on the float bits (the order of
-// non-negative floats), into an output the launcher zeroed; the others are
-// stored.  The maximum is exact, so the result does not depend on the order.
-// `staged` runs between the caller's two barriers: odd rows write, even rows read.
-__device__ __forceinline__ void stem_pool_rows(const float (&acc)[16][8], float (&h)[9][8]) {
+// pooled column pc (0..PX/2) stem columns 2 pc - 1 .. 2 pc + 1 (tile-relative).
+// Columns: each thread reduces its row's pixels to the windows it sees.
+// Rows: the odd rows go through shared memory to the even rows' threads, which
+// complete pooled rows 1..7.  Windows that reach into a neighbouring tile (the first
+// and last pooled rows and columns) are combined across tiles by an integer atomic
+// maximum on the float bits (the order of non-negative floats), into an output the
+// launcher zeroed; the others are stored.  The maximum is exact, so the result does
+// not depend on the order.
+template <int PX>
+__device__ __forceinline__ void stem_pool_rows(const float (&acc)[PX][8], float (&h)[PX / 2 + 1][8]) {
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     h[0][c] = fmaxf(acc[0][c], acc[1][c]);
 #pragma unroll
-    for (int k = 1; k < 8; ++k) h[k][c] = fmaxf(fmaxf(acc[2 * k - 1][c], acc[2 * k][c]), acc[2 * k + 1][c]);
-    h[8][c] = acc[15][c];
+    for (int k = 1; k < PX / 2; ++k) h[k][c] = fmaxf(fmaxf(acc[2 * k - 1][c], acc[2 * k][c]), acc[2 * k + 1][c]);
+    h[PX / 2][c] = acc[PX - 1][c];
   }
 }
 
-__global__ void __launch_bounds__(kStemThreads, 1) pq_stem7x7s2_kernel(const float* __restrict__ x,
-                                                                     const float* __restrict__ w,
-                                                                     float* __restrict__ y, float* __restrict__ pool,
-                                                                     int64_t N, int H, int W, int Ho, int Wo, int Hp,
-                                                                     int Wp, int relu) {
+template <int PX>
+__global__ void __launch_bounds__(kStemThreads, 1)
+    pq_stem7x7s2_kernel(const float* __restrict__ x, const float* __restrict__ w, float* __restrict__ y,
+                        float* __restrict__ pool, int64_t N, int H, int W, int Ho, int Wo, int Hp, int Wp, int relu,
+                        int vec) {
+  using T = StemTile<PX>;
   extern __shared__ float4 smem4[];
-  float* ws = reinterpret_cast<float*>(smem4);  // [147][2][16][4]
-  float* xs = ws + kStemTerms * kStemCout;      // the window [copy 4][parity 2][ci 3][row 37][16]
-  float* raw = xs + kStemXFloats;               // the next window [row 37][column 37][ci 3]
-  float* pstage = raw + kStemRawF;              // odd rows' pooled columns [8][9][128]
-  const int tiles_h = (Ho + kStemTH - 1) / kStemTH, tiles_w = (Wo + kStemTW - 1) / kStemTW;
-  const int64_t n_tiles = N * tiles_h * tiles_w;
-  // Tile t's window (element i = (row, column, channel) of the 37 x 37 x 3
-  // window, i = threadIdx.x + 256 e) into `raw` by 4-byte cp.async, zero-filled
-  // outside the image.
-  auto fetch = [&](int64_t t) {
-    const int tw = static_cast<int>(t % tiles_w);
+  float* ws = reinterpret_cast<float*>(smem4);  // [147][2][16][4], rows of kStemWF floats
+  const int grp = threadIdx.x / kStemGroup, tid = threadIdx.x % kStemGroup;
+  float* xs = ws + kStemTerms * kStemWF + grp * T::kGroupF;  // the window [parity 2][ci 3][row 37][position]
+  float* raw = xs + T::kXF;                                    // the next window [row 37][3 floats before, then columns x 3]
+  float* pstage = raw + T::kRawF;                              // odd rows' pooled columns [8][PX / 2 + 1][64]
+  const int tiles_h = (Ho + kStemTH - 1) / kStemTH, tiles_w = (Wo + PX - 1) / PX;
+  const int64_t n_items = 2 * N * tiles_h * tiles_w;  // (tile, channel half)
+  auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(kStemGroup) : "memory"); };
+  auto tile_at = [&](int64_t item, int64_t& n, int& th, int& tw) {
+    const int64_t t = item >> 1;
     const int64_t r = t / tiles_w;
-    const int th = static_cast<int>(r % tiles_h);
-    const int64_t n = r / tiles_h;
-    const int ih0 = th * kStemTH * kStemS - kStemP, iw0 = tw * kStemTW * kStemS - kStemP;
-#pragma unroll
-    for (int e = 0; e < kStemLoads; ++e) {
-      const int i = threadIdx.x + e * kStemThreads;
-      const int rr = i / (kStemIC * kStemCin), rem = i - rr * (kStemIC * kStemCin);
-      const int c = rem / kStemCin, ci = rem - c * kStemCin;
-      const int ih = ih0 + rr, iw = iw0 + c;
-      const bool valid = ih >= 0 && ih < H && iw >= 0 && iw < W;
-      if (i < kStemTileElems) cp_async4(raw + i, valid ? x + ((n * H + ih) * W + iw) * kStemCin + ci : x, valid);
+    tw = static_cast<int>(t - r * tiles_w);
+    n = r / tiles_h;
+    th = static_cast<int>(r - n * tiles_h);
+  };
+  // An item's window into `raw`, zero-filled outside the image: float i of a window
+  // row is float 3 + i of the raw row.
+  auto fetch = [&](int64_t item) {
+    int64_t n;
+    int th, tw;
+    tile_at(item, n, th, tw);
+    const int ih0 = th * kStemTH * kStemS - kStemP;
+    const int f0 = (tw * PX * kStemS - kStemP) * kStemCin - 3;  // the raw row's first float in the image row
+    const int row_f = W * kStemCin;
+    const float* img = x + n * H * row_f;
+    if (vec) {  // image rows are whole 16-byte pieces, and f0 is a multiple of 4 floats
+      for (int i = tid; i < kStemIR * T::kChunks; i += kStemGroup) {
+        const int rr = i / T::kChunks, c = i - rr * T::kChunks;
+        const int ih = ih0 + rr, f = f0 + 4 * c;
+        const bool valid = ih >= 0 && ih < H && f >= 0 && f < row_f;
+        cp_async16(raw + rr * T::kRawRowF + 4 * c, valid ? img + static_cast<int64_t>(ih) * row_f + f : x, valid);
+      }
+    } else {
+      for (int i = tid; i < T::kRawF; i += kStemGroup) {
+        const int rr = i / T::kRawRowF, c = i - rr * T::kRawRowF;
+        const int ih = ih0 + rr, f = f0 + c;
+        const bool valid = ih >= 0 && ih < H && f >= 0 && f < row_f;
+        cp_async4(raw + i, valid ? img + static_cast<int64_t>(ih) * row_f + f : x, valid);
+      }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  // The fetched window into the four shifted copies of its parity planes.
-  auto scatter = [&]() {
+  // The fetched window into its parity planes, one plane row (parity, channel, row) a
+  // thread: positions past the window's columns are never used.
+  auto split = [&]() {
+    for (int q = tid; q < 6 * kStemIR; q += kStemGroup) {
+      const int rr = q / 6, bc = q - rr * 6;  // bc = parity * 3 + channel
+      const float* src = raw + rr * T::kRawRowF + 3 + bc;
+      float4* dst = reinterpret_cast<float4*>(xs + bc * T::kPlaneF + rr * T::kRowF);
 #pragma unroll
-    for (int e = 0; e < kStemLoads; ++e) {
-      const int i = threadIdx.x + e * kStemThreads;
-      if (i < kStemTileElems) {
-        const float v = raw[i];
-        const int rr = i / (kStemIC * kStemCin), rem = i - rr * (kStemIC * kStemCin);
-        const int c = rem / kStemCin, ci = rem - c * kStemCin;
-        const int k0 = c >> 1;
-        float* dst = xs + ((c & 1) * kStemCin + ci) * kStemPlaneF + rr * kStemRowF + k0;
+      for (int k = 0; k < T::kRowF; k += 4) {
+        float v[4];
 #pragma unroll
-        for (int sh = 0; sh < 4; ++sh)
-          if (k0 - sh >= 0 && k0 - sh < kStemRowF) dst[sh * kStemCopyF - sh] = v;
+        for (int e = 0; e < 4; ++e) v[e] = 3 + 6 * (k + e) + 2 < T::kRawRowF ? src[6 * (k + e)] : 0.0f;
+        dst[k / 4] = make_float4(v[0], v[1], v[2], v[3]);
       }
     }
   };
-  int64_t t = blockIdx.x;
-  if (t < n_tiles) fetch(t);
-  // weights [Cout][147] to [147][2][16][4]: channel co = 8 g + 4 h + k at
-  // term * 128 + h * 64 + g * 4 + k (consecutive threads write consecutive words)
+  const int64_t step = 2 * static_cast<int64_t>(gridDim.x);
+  int64_t item = static_cast<int64_t>(grp) * gridDim.x + blockIdx.x;
+  if (item < n_items) fetch(item);
+  // weights [Cout][147] to [147][2][16][4]: channel co = 8 g + 4 h + k of a term at
+  // h * 64 + g * 4 + k
   for (int i = threadIdx.x; i < kStemTerms * kStemCout; i += kStemThreads) {
-    const int term = i >> 7, rem = i & 127;
-    const int h = rem >> 6, g = (rem >> 2) & 15, k = rem & 3;
-    ws[i] = w[(g * 8 + h * 4 + k) * kStemTerms + term];
+    const int co = i / kStemTerms, term = i - co * kStemTerms;
+    cp_async4(ws + term * kStemWF + ((co >> 2) & 1) * 64 + (co >> 3) * 4 + (co & 3), w + i, true);
   }
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-  __syncthreads();  // the first window landed
-  scatter();
-  __syncthreads();  // the first window's copies and the weights visible to all threads
-  const int cg = threadIdx.x & 15, r = threadIdx.x >> 4;  // channel group, tile row
-  const float* wthr = ws + cg * 4;
-  const float* xthr = xs + (2 * r) * kStemRowF;
-  for (; t < n_tiles; t += gridDim.x) {
-    const bool more = t + gridDim.x < n_tiles;
-    if (more) fetch(t + gridDim.x);  // in flight during the FMAs
+  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+  __syncthreads();  // the first windows and the weights landed
+  split();
+  group_sync();
+  // The second group's first FMAs wait for the first group to be two sevenths through
+  // its first tile (where a second tile follows).
+  const bool stagger = gridDim.x + blockIdx.x + step < n_items;
+  if (stagger && grp == 1) asm volatile("bar.sync 3, %0;" ::"n"(kStemThreads) : "memory");
+  bool first = true;
+  const int cg = tid & 7, r = tid >> 3;  // channel group of the half, tile row
+  const float* xthr = xs + (2 * r) * T::kRowF;
+  for (; item < n_items; item += step, first = false) {
+    const int ch = static_cast<int>(item & 1) * kStemHalf + cg * 8;  // first channel
+    const float* wthr = ws + (ch >> 3) * 4;
+    const bool more = item + step < n_items;
+    if (more) fetch(item + step);  // in flight during the FMAs
     // the sums of pixel j, channels 2 k and 2 k + 1, as one 64-bit register pair
-    unsigned long long a2[16][4];
+    unsigned long long a2[PX][4];
 #pragma unroll
-    for (int j = 0; j < 16; ++j)
+    for (int j = 0; j < PX; ++j)
 #pragma unroll
       for (int k = 0; k < 4; ++k) a2[j][k] = 0ull;
 #pragma unroll 1
     for (int kh = 0; kh < kStemK; ++kh) {
-      const float* xk = xthr + kh * kStemRowF;
-      const float* wk = wthr + kh * (kStemK * kStemCin) * kStemCout;
+      if (stagger && first && grp == 0 && kh == 2) asm volatile("bar.arrive 3, %0;" ::"n"(kStemThreads) : "memory");
+      const float* xk = xthr + kh * T::kRowF;
+      const float* wk = wthr + kh * (kStemK * kStemCin) * kStemWF;
 #pragma unroll
       for (int kw = 0; kw < kStemK; ++kw) {
+        constexpr int kQ = PX / 4 + 1;
+        const int sh = kw >> 1;
 #pragma unroll
         for (int ci = 0; ci < kStemCin; ++ci) {
-          const float4* xp =
-              reinterpret_cast<const float4*>(xk + (kw >> 1) * kStemCopyF + ((kw & 1) * kStemCin + ci) * kStemPlaneF);
-          const float4 x0 = xp[0], x1 = xp[1], x2 = xp[2], x3 = xp[3];
-          const float* wt = wk + (kw * kStemCin + ci) * kStemCout;
+          const float4* xp = reinterpret_cast<const float4*>(xk + ((kw & 1) * kStemCin + ci) * T::kPlaneF);
+          float xv[4 * kQ];
+#pragma unroll
+          for (int q = 0; q < kQ; ++q) {
+            if (q == kQ - 1 && sh == 0) break;
+            const float4 v = xp[q];
+            xv[4 * q] = v.x;
+            xv[4 * q + 1] = v.y;
+            xv[4 * q + 2] = v.z;
+            xv[4 * q + 3] = v.w;
+          }
+          const float* wt = wk + (kw * kStemCin + ci) * kStemWF;
           // the weight pairs (channels 2 k, 2 k + 1) as they lie in shared memory
           const ulonglong2 wa = *reinterpret_cast<const ulonglong2*>(wt);
           const ulonglong2 wb = *reinterpret_cast<const ulonglong2*>(wt + 64);
-          const float xv[16] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w,
-                                x2.x, x2.y, x2.z, x2.w, x3.x, x3.y, x3.z, x3.w};
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const unsigned long long xx = f32x2_pair(xv[j], xv[j]);
+          for (int j = 0; j < PX; ++j) {
+            const unsigned long long xx = f32x2_pair(xv[sh + j], xv[sh + j]);
             ffma2(a2[j][0], xx, wa.x);
             ffma2(a2[j][1], xx, wa.y);
             ffma2(a2[j][2], xx, wb.x);
@@ -284,19 +325,18 @@ __global__ void __launch_bounds__(kStemThreads, 1) pq_stem7x7s2_kernel(const flo
         }
       }
     }
-    float acc[16][8];
+    float acc[PX][8];
 #pragma unroll
-    for (int j = 0; j < 16; ++j)
+    for (int j = 0; j < PX; ++j)
 #pragma unroll
       for (int k = 0; k < 4; ++k) f32x2_unpair(a2[j][k], acc[j][2 * k], acc[j][2 * k + 1]);
-    const int tw = static_cast<int>(t % tiles_w);
-    const int64_t rt = t / tiles_w;
-    const int th = static_cast<int>(rt % tiles_h);
-    const int64_t n = rt / tiles_h;
+    int64_t n;
+    int th, tw;
+    tile_at(item, n, th, tw);
     const int oh = th * kStemTH + r;
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const bool in_out = oh < Ho && tw * kStemTW + j < Wo;
+    for (int j = 0; j < PX; ++j) {
+      const bool in_out = oh < Ho && tw * PX + j < Wo;
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
         if (relu) acc[j][c] = fmaxf(acc[j][c], 0.0f);
@@ -305,35 +345,35 @@ __global__ void __launch_bounds__(kStemThreads, 1) pq_stem7x7s2_kernel(const flo
         if (pool != nullptr && !in_out) acc[j][c] = 0.0f;
       }
       if (y != nullptr && in_out) {
-        float4* yp = reinterpret_cast<float4*>(y + ((n * Ho + oh) * Wo + tw * kStemTW + j) * kStemCout + cg * 8);
+        float4* yp = reinterpret_cast<float4*>(y + ((n * Ho + oh) * Wo + tw * PX + j) * kStemCout + ch);
         yp[0] = make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
         yp[1] = make_float4(acc[j][4], acc[j][5], acc[j][6], acc[j][7]);
       }
     }
-    // Every warp is done with this window and, from the previous tile, with the
-    // pooling stage, and every thread's copies of the next window have landed.
+    // Every warp of the group is done with this window and, from the previous item,
+    // with the pooling stage, and every thread's copies of the next window have landed.
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();
-    if (more) scatter();
+    group_sync();
+    if (more) split();
     if (pool != nullptr) {
-      float h[9][8];
-      stem_pool_rows(acc, h);
+      float h[T::kPC][8];
+      stem_pool_rows<PX>(acc, h);
       if (r & 1) {
 #pragma unroll
-        for (int pc = 0; pc < 9; ++pc) {
-          float4* d = reinterpret_cast<float4*>(pstage + (r >> 1) * kStemPoolRowF + pc * kStemCout + cg * 8);
+        for (int pc = 0; pc < T::kPC; ++pc) {
+          float4* d = reinterpret_cast<float4*>(pstage + (r >> 1) * T::kPoolRowF + pc * kStemHalf + cg * 8);
           d[0] = make_float4(h[pc][0], h[pc][1], h[pc][2], h[pc][3]);
           d[1] = make_float4(h[pc][4], h[pc][5], h[pc][6], h[pc][7]);
         }
       }
-      __syncthreads();  // the odd rows staged and the next window's copies written
+      group_sync();  // the odd rows staged and the next window split
       if ((r & 1) == 0 || r == kStemTH - 1) {
         const int pr = (r + 1) >> 1;  // even rows: r / 2; the last row: pooled row 8
         const int64_t pi = static_cast<int64_t>(th) * (kStemTH / 2) + pr;
         if (pi < Hp) {
 #pragma unroll
-          for (int pc = 0; pc < 9; ++pc) {
-            const int pj = tw * (kStemTW / 2) + pc;
+          for (int pc = 0; pc < T::kPC; ++pc) {
+            const int pj = tw * (PX / 2) + pc;
             if (pj >= Wp) continue;
             float v[8];
 #pragma unroll
@@ -343,14 +383,15 @@ __global__ void __launch_bounds__(kStemThreads, 1) pq_stem7x7s2_kernel(const flo
               for (int rr = -1; rr <= 1; rr += 2) {
                 const int ro = r + rr;
                 if (ro < 0) continue;
-                const float4* sp = reinterpret_cast<const float4*>(pstage + (ro >> 1) * kStemPoolRowF + pc * kStemCout + cg * 8);
+                const float4* sp =
+                    reinterpret_cast<const float4*>(pstage + (ro >> 1) * T::kPoolRowF + pc * kStemHalf + cg * 8);
                 const float4 pa = sp[0], pb = sp[1];
                 v[0] = fmaxf(v[0], pa.x); v[1] = fmaxf(v[1], pa.y); v[2] = fmaxf(v[2], pa.z); v[3] = fmaxf(v[3], pa.w);
                 v[4] = fmaxf(v[4], pb.x); v[5] = fmaxf(v[5], pb.y); v[6] = fmaxf(v[6], pb.z); v[7] = fmaxf(v[7], pb.w);
               }
             }
-            float* dst = pool + ((n * Hp + pi) * Wp + pj) * kStemCout + cg * 8;
-            const bool whole = pr >= 1 && pr <= kStemTH / 2 - 1 && pc >= 1 && pc <= 7;
+            float* dst = pool + ((n * Hp + pi) * Wp + pj) * kStemCout + ch;
+            const bool whole = pr >= 1 && pr <= kStemTH / 2 - 1 && pc >= 1 && pc <= PX / 2 - 1;
             if (whole) {
               reinterpret_cast<float4*>(dst)[0] = make_float4(v[0], v[1], v[2], v[3]);
               reinterpret_cast<float4*>(dst)[1] = make_float4(v[4], v[5], v[6], v[7]);
@@ -362,7 +403,7 @@ __global__ void __launch_bounds__(kStemThreads, 1) pq_stem7x7s2_kernel(const flo
         }
       }
     } else {
-      __syncthreads();  // the next window's copies written
+      group_sync();  // the next window split
     }
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -561,17 +602,40 @@ int64_t out_dim(int64_t n, int k, int s, int p) { return (n + 2 * p - k) / s + 1
 bool aligned16(const void* ptr) { return (reinterpret_cast<uintptr_t>(ptr) & 15u) == 0; }
 
 }  // namespace
-// The stem kernel's dynamic shared memory above the default limit, once per
-// process (the network runs on one device).
-bool stem_smem_attribute() {
+// Launch of the stem kernel (pool and y may be NULL); 0 on success.  Tiles of 8 columns
+// while the ones of 16 give the chip's groups less than 1.5 items each: half the time of
+// an item, at more loads and border windows for each FMA (1, 2, 4, 6, 8 images of
+// 224x224: 18.4, 25.3, 42.0, 54.8, 75.2 us; with 16: 19.6, 30.6, 44.6, 54.2, 76.5; 128
+// images 1022 and 984).  The dynamic shared memory above
+// the default limit is allowed once per instance and process (the network runs on one
+// device).
+template <int PX>
+int launch_stem_px(const float* x, const float* w, float* y, float* pool, int64_t N, int H, int W, int Ho, int Wo, int Hp,
+                   int Wp, int relu, int sms, cudaStream_t stream) {
   static bool done = false;
   if (!done) {
-    if (cudaFuncSetAttribute(pq_stem7x7s2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kStemSmem)) != cudaSuccess)
-      return false;
+    if (cudaFuncSetAttribute(pq_stem7x7s2_kernel<PX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(StemTile<PX>::kSmem)) != cudaSuccess)
+      return -1;
     done = true;
   }
-  return true;
+  const int64_t items = 2 * N * ((Ho + kStemTH - 1) / kStemTH) * ((Wo + PX - 1) / PX);
+  const unsigned grid = static_cast<unsigned>(items < sms ? items : sms);
+  const int vec = (static_cast<int64_t>(W) * kStemCin) % 4 == 0 && aligned16(x);
+  pq_stem7x7s2_kernel<PX><<<grid, kStemThreads, StemTile<PX>::kSmem, stream>>>(x, w, y, pool, N, H, W, Ho, Wo, Hp, Wp,
+                                                                             relu, vec);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+int launch_stem(const float* x, const float* w, float* y, float* pool, int64_t N, int H, int W, int Ho, int Wo, int Hp,
+                int Wp, int relu, cudaStream_t stream) {
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t tiles = N * ((Ho + kStemTH - 1) / kStemTH) * ((Wo + 15) / 16);
+  if (2 * tiles <= 3 * sms)
+    return launch_stem_px<8>(x, w, y, pool, N, H, W, Ho, Wo, Hp, Wp, relu, sms, stream);
+  return launch_stem_px<16>(x, w, y, pool, N, H, W, Ho, Wo, Hp, Wp, relu, sms, stream);
 }
 
 }  // namespace pq
@@ -592,15 +656,10 @@ pq_status palquant_conv2d_f32(const float* x_dev, const float* w_dev, float* y_d
   auto s = static_cast<cudaStream_t>(stream);
   if (k == pq::kStemK && stride == pq::kStemS && pad == pq::kStemP && Cin == pq::kStemCin && Cout == pq::kStemCout &&
       pq::aligned16(y_dev)) {
-    if (!pq::stem_smem_attribute()) return PQ_ECUDA;
-    const int64_t tiles = N * ((Ho + pq::kStemTH - 1) / pq::kStemTH) * ((Wo + pq::kStemTW - 1) / pq::kStemTW);
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const unsigned grid = static_cast<unsigned>(tiles < static_cast<int64_t>(sms) ? tiles : sms);
-    pq::pq_stem7x7s2_kernel<<<grid, pq::kStemThreads, pq::kStemSmem, s>>>(
-        x_dev, w_dev, y_dev, nullptr, N, H, W, static_cast<int>(Ho), static_cast<int>(Wo), 0, 0, relu);
-    return cudaGetLastError() == cudaSuccess ? PQ_OK : PQ_ECUDA;
+    return pq::launch_stem(x_dev, w_dev, y_dev, nullptr, N, H, W, static_cast<int>(Ho), static_cast<int>(Wo), 0, 0, relu,
+                           s) == 0
+               ? PQ_OK
+               : PQ_ECUDA;
   }
   if (wbytes <= 96 * 1024) {
     static bool attr_set = false;
@@ -629,19 +688,13 @@ pq_status palquant_stem_pool_f32(const float* x_dev, const float* w_dev, float* 
   const int64_t Hp = pq::out_dim(Ho, 3, 2, 1), Wp = pq::out_dim(Wo, 3, 2, 1);
   if (N == 0) return PQ_OK;
   auto s = static_cast<cudaStream_t>(stream);
-  if (!pq::stem_smem_attribute()) return PQ_ECUDA;
   // border windows are combined by atomic maxima over non-negative values: start from 0
   if (cudaMemsetAsync(pool_dev, 0, static_cast<size_t>(N * Hp * Wp * Cout) * sizeof(float), s) != cudaSuccess)
     return PQ_ECUDA;
-  const int64_t tiles = N * ((Ho + pq::kStemTH - 1) / pq::kStemTH) * ((Wo + pq::kStemTW - 1) / pq::kStemTW);
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const unsigned grid = static_cast<unsigned>(tiles < static_cast<int64_t>(sms) ? tiles : sms);
-  pq::pq_stem7x7s2_kernel<<<grid, pq::kStemThreads, pq::kStemSmem, s>>>(
-      x_dev, w_dev, stem_dev, pool_dev, N, H, W, static_cast<int>(Ho), static_cast<int>(Wo), static_cast<int>(Hp),
-      static_cast<int>(Wp), 1);
-  return cudaGetLastError() == cudaSuccess ? PQ_OK : PQ_ECUDA;
+  return pq::launch_stem(x_dev, w_dev, stem_dev, pool_dev, N, H, W, static_cast<int>(Ho), static_cast<int>(Wo),
+                         static_cast<int>(Hp), static_cast<int>(Wp), 1, s) == 0
+             ? PQ_OK
+             : PQ_ECUDA;
 }
 
 pq_status palquant_maxpool2d_f32(const float* x_dev, float* y_dev, int64_t N, int32_t H, int32_t W, int32_t C,

@@ -247,3 +247,23 @@ def test_paper_placement_gpu_calibration_matches_oracle():
         assert np.all(d <= 1), k
     for k in ref:
         assert np.allclose(got[k], ref[k], rtol=1e-3), k
+
+
+# Tiles of 16 columns (many images) and of 8 (few), rows whose 16-byte pieces are aligned
+# and not, several items per group of the kernel.
+@pytest.mark.parametrize("N,H,W", [(230, 18, 21), (231, 20, 36), (3, 41, 67), (1, 7, 4), (40, 33, 40)])
+def test_stem_pool_tile_widths_match_oracle(N, H, W):
+    import oracle
+    from paper_2208_01944_gb300 import binding as B
+
+    gen = synth.generator(300 + N + H + W)
+    x = synth.normal((N, H, W, 3), gen)
+    w = synth.normal((128, 7, 7, 3), gen, 0.1)
+    stem = oracle.conv2d_f32(x, w, 2, 3, True)
+    ref = oracle.maxpool_f32(stem, 3, 2, 1)
+    pool = torch.full(ref.shape, float("nan"), dtype=torch.float32, device="cuda")
+    st = torch.full(stem.shape, float("nan"), dtype=torch.float32, device="cuda")
+    B.palquant_stem_pool_f32(torch.from_numpy(x).cuda(), torch.from_numpy(w).cuda(), st, pool, N, H, W, 128)
+    assert B.palquant_sync_check() == B.PQ_OK
+    assert np.array_equal(pool.cpu().numpy(), ref)
+    assert np.array_equal(st.cpu().numpy(), stem)
