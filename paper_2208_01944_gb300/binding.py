@@ -155,26 +155,52 @@ lib = _load()
 
 
 # ----------------------------------------------------------------- marshalling
+# A call's own time is mostly its launch; the marshalling around it is kept to a few
+# attribute reads (a pointwise layer call took 16 us on the host, 12 of them here: torch's
+# Stream object, its availability check and numpy's ctypes object; now 7).
 def _ptr(obj):
     """Device or host address of a tensor / array / int (None -> NULL)."""
     if obj is None:
         return None
+    address = getattr(obj, "data_ptr", None)
+    if address is not None:
+        assert obj.is_contiguous(), "tensors passed to libpalquant must be contiguous"
+        return address()
     if isinstance(obj, int):
         return obj
     if isinstance(obj, np.ndarray):
-        assert obj.flags["C_CONTIGUOUS"]
-        return obj.ctypes.data
-    if hasattr(obj, "data_ptr"):
-        assert obj.is_contiguous(), "tensors passed to libpalquant must be contiguous"
-        return obj.data_ptr()
+        assert obj.flags.c_contiguous
+        return obj.__array_interface__["data"][0]
     raise TypeError(f"cannot pass {type(obj)} as a pointer")
+
+
+def _floats(a):
+    """Host floats as a C argument (None -> NULL); it keeps the array alive."""
+    if a is None:
+        return None
+    f = _f32(a)
+    if f.size and f.flags.writeable:
+        return ctypes.byref(ctypes.c_float.from_buffer(f))
+    f = np.array(f if f.size else [0.0], dtype=np.float32)  # read-only or empty: a copy of its own
+    return ctypes.byref(ctypes.c_float.from_buffer(f))
+
+
+def _current_stream():
+    """Raw handle of torch's current stream on its current device (None without a GPU)."""
+    global _current_stream
+    import torch
+
+    if not torch.cuda.is_available():
+        return None
+    handle = torch.cuda.current_stream().cuda_stream  # initialises CUDA in this process
+    get_device, get_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+    _current_stream = lambda: get_stream(get_device())  # noqa: E731  (from now on)
+    return handle
 
 
 def _stream(stream):
     if stream is None:
-        import torch
-
-        return torch.cuda.current_stream().cuda_stream if torch.cuda.is_available() else None
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -289,8 +315,7 @@ def palquant_unpack_weight_codes_host(packed_host, d: LayerDesc) -> np.ndarray:
 
 
 def palquant_quantize_act(x_dev, q_dev, N, H, W, G, Cg, bits, inv_s, code_format=PQ_CODES_INT8, stream=None):
-    inv = _f32(inv_s)
-    _check(lib.palquant_quantize_act(_ptr(x_dev), _ptr(q_dev), N, H, W, G, Cg, bits, code_format, _ptr(inv),
+    _check(lib.palquant_quantize_act(_ptr(x_dev), _ptr(q_dev), N, H, W, G, Cg, bits, code_format, _floats(inv_s),
                                      _stream(stream)), "palquant_quantize_act")
 
 
@@ -301,29 +326,23 @@ def palquant_group_conv(q_dev, w_packed_dev, acc_dev, d: LayerDesc, stream=None)
 
 def palquant_layer_fused(q_dev, w_packed_dev, d: LayerDesc, m_out, m_req=None, shuf=None, shortcut_dev=None,
                          acc_out_dev=None, y_out_dev=None, q_out_dev=None, stream=None):
-    mo = None if m_out is None else _f32(m_out)
-    mr = None if m_req is None else _f32(m_req)
-    _check(lib.palquant_layer_fused(_ptr(q_dev), _ptr(w_packed_dev), ctypes.byref(d), _ptr(mo), _ptr(mr),
+    _check(lib.palquant_layer_fused(_ptr(q_dev), _ptr(w_packed_dev), ctypes.byref(d), _floats(m_out), _floats(m_req),
                                     shuf or shuffle(1, 1), _ptr(shortcut_dev), _ptr(acc_out_dev), _ptr(y_out_dev),
                                     _ptr(q_out_dev), _stream(stream)), "palquant_layer_fused")
 
 
 def palquant_quantize_layer_fused(x_dev, inv_s, w_packed_dev, d: LayerDesc, m_out, m_req=None, shuf=None,
                                   shortcut_dev=None, acc_out_dev=None, y_out_dev=None, q_out_dev=None, stream=None):
-    inv = _f32(inv_s)
-    mo = None if m_out is None else _f32(m_out)
-    mr = None if m_req is None else _f32(m_req)
-    _check(lib.palquant_quantize_layer_fused(_ptr(x_dev), _ptr(inv), _ptr(w_packed_dev), ctypes.byref(d), _ptr(mo),
-                                             _ptr(mr), shuf or shuffle(1, 1), _ptr(shortcut_dev), _ptr(acc_out_dev),
+    _check(lib.palquant_quantize_layer_fused(_ptr(x_dev), _floats(inv_s), _ptr(w_packed_dev), ctypes.byref(d),
+                                             _floats(m_out), _floats(m_req), shuf or shuffle(1, 1), _ptr(shortcut_dev), _ptr(acc_out_dev),
                                              _ptr(y_out_dev), _ptr(q_out_dev), _stream(stream)),
            "palquant_quantize_layer_fused")
 
 
 def palquant_cyclic_shuffle_module(q_dev, w_packed_dev, d: LayerDesc, m_out, m_req=None, shift=1, x_dev=None,
                                    z_out_dev=None, q_out_dev=None, stream=None):
-    mo = None if m_out is None else _f32(m_out)
-    mr = None if m_req is None else _f32(m_req)
-    _check(lib.palquant_cyclic_shuffle_module(_ptr(q_dev), _ptr(w_packed_dev), ctypes.byref(d), _ptr(mo), _ptr(mr),
+    _check(lib.palquant_cyclic_shuffle_module(_ptr(q_dev), _ptr(w_packed_dev), ctypes.byref(d), _floats(m_out),
+                                              _floats(m_req),
                                               int(shift), _ptr(x_dev), _ptr(z_out_dev), _ptr(q_out_dev),
                                               _stream(stream)), "palquant_cyclic_shuffle_module")
 
@@ -419,8 +438,7 @@ def palquant_pack_weights_odd_host(w_host, d: LayerDesc, u) -> np.ndarray:
 # ---------------------------------------------------------------- quantisation-aware training
 def palquant_fake_quant_forward(x_dev, xhat_dev, P, G, Cg, bits, kind, l, u, stream=None) -> None:
     """Fake quantisation with learned per-group bounds (Eq. 2-3); kind 0 activations, 1 weights."""
-    lf, uf = _f32(l), _f32(u)
-    _check(lib.palquant_fake_quant_forward(_ptr(x_dev), _ptr(xhat_dev), P, G, Cg, bits, kind, _ptr(lf), _ptr(uf),
+    _check(lib.palquant_fake_quant_forward(_ptr(x_dev), _ptr(xhat_dev), P, G, Cg, bits, kind, _floats(l), _floats(u),
                                            _stream(stream)), "palquant_fake_quant_forward")
 
 
@@ -431,28 +449,23 @@ def palquant_fake_quant_scratch_bytes(P, G, Cg) -> int:
 def palquant_fake_quant_backward(x_dev, dy_dev, dx_dev, dl_dev, du_dev, P, G, Cg, bits, kind, l, u, scratch_dev,
                                  scratch_bytes, stream=None) -> None:
     """Straight-through backward: dx (fp32) and the per-group gradients of l and u (G doubles each, device)."""
-    lf, uf = _f32(l), _f32(u)
     _check(lib.palquant_fake_quant_backward(_ptr(x_dev), _ptr(dy_dev), _ptr(dx_dev), _ptr(dl_dev), _ptr(du_dev), P, G,
-                                            Cg, bits, kind, _ptr(lf), _ptr(uf), _ptr(scratch_dev), scratch_bytes,
+                                            Cg, bits, kind, _floats(l), _floats(u), _ptr(scratch_dev), scratch_bytes,
                                             _stream(stream)), "palquant_fake_quant_backward")
 
 
 # ---------------------------------------------------------------- learned bounds at inference
 def palquant_quantize_act_lu(x_dev, q_dev, N, H, W, G, Cg, bits, l, u, code_format=PQ_CODES_INT8, stream=None):
     """Activation codes with learned per-group bounds l < u (the training forward's codes)."""
-    lf, uf = _f32(l), _f32(u)
-    _check(lib.palquant_quantize_act_lu(_ptr(x_dev), _ptr(q_dev), N, H, W, G, Cg, bits, code_format, _ptr(lf),
-                                        _ptr(uf), _stream(stream)), "palquant_quantize_act_lu")
+    _check(lib.palquant_quantize_act_lu(_ptr(x_dev), _ptr(q_dev), N, H, W, G, Cg, bits, code_format, _floats(l),
+                                        _floats(u), _stream(stream)), "palquant_quantize_act_lu")
 
 
 def palquant_quantize_layer_fused_lu(x_dev, l, u, w_packed_dev, d: LayerDesc, m_out, m_req=None, shuf=None,
                                      shortcut_dev=None, acc_out_dev=None, y_out_dev=None, q_out_dev=None,
                                      stream=None):
     """Quantise-on-load with learned per-group bounds l < u, then the layer."""
-    lf, uf = _f32(l), _f32(u)
-    mo = None if m_out is None else _f32(m_out)
-    mr = None if m_req is None else _f32(m_req)
-    _check(lib.palquant_quantize_layer_fused_lu(_ptr(x_dev), _ptr(lf), _ptr(uf), _ptr(w_packed_dev), ctypes.byref(d),
-                                                _ptr(mo), _ptr(mr), shuf or shuffle(1, 1), _ptr(shortcut_dev),
+    _check(lib.palquant_quantize_layer_fused_lu(_ptr(x_dev), _floats(l), _floats(u), _ptr(w_packed_dev),
+                                                ctypes.byref(d), _floats(m_out), _floats(m_req), shuf or shuffle(1, 1), _ptr(shortcut_dev),
                                                 _ptr(acc_out_dev), _ptr(y_out_dev), _ptr(q_out_dev), _stream(stream)),
            "palquant_quantize_layer_fused_lu")

@@ -135,7 +135,7 @@ struct Tile {
 
 constexpr int kPlanSMs = 152;  // SMs the planner counts on
 
-pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, std::vector<Phase>* phases_out,
+pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub,
                     bool quant_in = false, bool direct_out = false, bool shortcut = false,
                     const Tile* tile = nullptr) {
   // Epilogue staging per warp: 32 rows of up to 32 fp32/int32 values (128 bytes,
@@ -375,11 +375,11 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
       }
       const bool differs = fast.MT != 0 && (fast.MT != best.MT || fast.nsub != 1);
       if (differs) {
-        pq_status base = plan_conv(d, P, pub, phases_out, quant_in, direct_out, shortcut, &best);
+        pq_status base = plan_conv(d, P, pub, quant_in, direct_out, shortcut, &best);
         if (base != PQ_OK) return base;
         ConvParams pf;
         pq_conv_plan pubf;
-        if (plan_conv(d, &pf, &pubf, nullptr, quant_in, direct_out, shortcut, &fast) == PQ_OK) {
+        if (plan_conv(d, &pf, &pubf, quant_in, direct_out, shortcut, &fast) == PQ_OK) {
           if (P) *P = pf;
           if (pub) *pub = pubf;
         }
@@ -651,8 +651,39 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub, st
   plan.work_items = p.items;
   if (pub) *pub = plan;
   if (P) *P = p;
-  if (phases_out) *phases_out = phases;
   return PQ_OK;
+}
+
+// plan_conv of a layer call, remembered by value: a program calls the same few layers
+// again and again, and planning one costs about 1 us of its 4 us on the host.  A fixed
+// number of plans per host thread, given back with the thread.
+pq_status plan_call(const pq_layer_desc* d, ConvParams* P, bool quant_in, bool direct_out, bool shortcut) {
+  struct Slot {
+    bool used = false;
+    pq_layer_desc d;
+    int mode;
+    pq_status st;
+    ConvParams p;
+  };
+  constexpr int kSlots = 16;
+  thread_local Slot slots[kSlots];
+  pq_layer_desc key = *d;
+  key.flags = 0;  // no part of a plan
+  const int mode = (quant_in ? 1 : 0) | (direct_out ? 2 : 0) | (shortcut ? 4 : 0);
+  static_assert(sizeof(pq_layer_desc) % sizeof(int32_t) == 0, "a descriptor is 32-bit words without padding");
+  uint32_t h = static_cast<uint32_t>(mode) + 2166136261u;
+  int32_t word[sizeof(pq_layer_desc) / sizeof(int32_t)];
+  std::memcpy(word, &key, sizeof(key));
+  for (int32_t w : word) h = (h ^ static_cast<uint32_t>(w)) * 16777619u;
+  Slot& s = slots[(h ^ (h >> 16)) % kSlots];
+  if (!s.used || s.mode != mode || std::memcmp(&s.d, &key, sizeof(key)) != 0) {
+    s.used = true;
+    s.d = key;
+    s.mode = mode;
+    s.st = plan_conv(&key, &s.p, nullptr, quant_in, direct_out, shortcut);
+  }
+  if (s.st == PQ_OK) *P = s.p;
+  return s.st;
 }
 
 // ---------------------------------------------------------------------------
@@ -974,13 +1005,12 @@ pq_status layer_fused_impl(const void* q_dev, const void* w_packed_dev, const pq
       !aligned16(q_out_dev) || !aligned16(shortcut_dev))
     return PQ_EINVAL;
   ConvParams p;
-  std::vector<Phase> phases;
   // Channel-blocked codes as the only output are stored from registers (the
   // per-channel scatter of the channel shuffle is unstaged too).
   const bool direct_out =
       acc_out_dev == nullptr && y_out_dev == nullptr && shortcut_dev == nullptr && d->code_format != PQ_CODES_INT8;
   const bool quant_in = inv_s_in != nullptr || l_in != nullptr;
-  st = plan_conv(d, &p, nullptr, &phases, quant_in, direct_out, shortcut_dev != nullptr);
+  st = plan_call(d, &p, quant_in, direct_out, shortcut_dev != nullptr);
   if (st != PQ_OK) return st;
   if (l_in != nullptr) {
     // learned bounds: the training forward's codes (sat((x - l) * fl(1/fl(u - l))) * Qp, rounded)
@@ -1155,7 +1185,7 @@ pq_status palquant_epilogue_scales(int32_t G, const float* s_w_host, const float
 
 size_t palquant_packed_weight_bytes(const pq_layer_desc* d) {
   ConvParams p;
-  if (plan_conv(d, &p, nullptr, nullptr) != PQ_OK) return 0;
+  if (plan_conv(d, &p, nullptr) != PQ_OK) return 0;
   return packed_weight_bytes_of(d, p);
 }
 
@@ -1163,7 +1193,7 @@ pq_status palquant_pack_weight_codes_host(const int8_t* wq_host, const pq_layer_
                                           size_t packed_bytes) {
   if (wq_host == nullptr || packed_host == nullptr) return PQ_EINVAL;
   ConvParams p;
-  pq_status st = plan_conv(d, &p, nullptr, nullptr);
+  pq_status st = plan_conv(d, &p, nullptr);
   if (st != PQ_OK) return st;
   const size_t elems = static_cast<size_t>(d->G) * d->Cout_g * weight_taps(d) * d->Cin_g;
   if (packed_bytes < packed_weight_bytes_of(d, p)) return PQ_EINVAL;
@@ -1177,7 +1207,7 @@ pq_status palquant_pack_weight_codes_host(const int8_t* wq_host, const pq_layer_
 pq_status palquant_unpack_weight_codes_host(const void* packed_host, const pq_layer_desc* d, int8_t* wq_host) {
   if (packed_host == nullptr || wq_host == nullptr) return PQ_EINVAL;
   ConvParams p;
-  pq_status st = plan_conv(d, &p, nullptr, nullptr);
+  pq_status st = plan_conv(d, &p, nullptr);
   if (st != PQ_OK) return st;
   const uint8_t* in = static_cast<const uint8_t*>(packed_host);
   const int kwr = d->kw * wslices_of(d);
@@ -1216,7 +1246,7 @@ pq_status palquant_pack_weights_odd_host(const float* w_host, const pq_layer_des
                                         void* packed_host, size_t packed_bytes) {
   if (w_host == nullptr || u_host == nullptr || packed_host == nullptr) return PQ_EINVAL;
   ConvParams p;
-  pq_status st = plan_conv(d, &p, nullptr, nullptr);
+  pq_status st = plan_conv(d, &p, nullptr);
   if (st != PQ_OK) return st;
   if (wslices_of(d) != 1) return PQ_EINVAL;  // float weights belong to plain layers
   const size_t per_group = static_cast<size_t>(d->Cout_g) * d->kh * d->kw * d->Cin_g;
@@ -1413,7 +1443,7 @@ pq_status palquant_bitsplit_desc(const pq_layer_desc* d, int32_t bits_b, pq_laye
   pq_status st = bitsplit_layer(d, bits_b, &t, &Ga, &Gw);
   if (st != PQ_OK) return st;
   ConvParams p;
-  st = plan_conv(&t, &p, nullptr, nullptr);
+  st = plan_conv(&t, &p, nullptr);
   if (st != PQ_OK) return st;
   *out = t;
   return PQ_OK;
@@ -1433,7 +1463,7 @@ pq_status palquant_bitsplit_pack_weight_codes_host(const int8_t* wq_host, const 
   pq_status st = bitsplit_layer(d, bits_b, &t, &Ga, &Gw);
   if (st != PQ_OK) return st;
   ConvParams p;
-  st = plan_conv(&t, &p, nullptr, nullptr);
+  st = plan_conv(&t, &p, nullptr);
   if (st != PQ_OK) return st;
   const size_t need = static_cast<size_t>(t.G) * t.Cout_g * t.kh * t.kw * t.Cin_g;
   if (packed_bytes < need) return PQ_EINVAL;
@@ -1519,7 +1549,7 @@ pq_status palquant_watchdog_selftest(uint64_t limit_ns, pq_stream_t stream) {
 
 pq_status palquant_conv_plan(const pq_layer_desc* d, pq_conv_plan* plan) {
   if (plan == nullptr) return PQ_EINVAL;
-  const pq_status st = plan_conv(d, nullptr, plan, nullptr);
+  const pq_status st = plan_conv(d, nullptr, plan);
   if (st == PQ_OK) plan->pointwise = plan_pointwise(d, nullptr) ? 1 : 0;
   return st;
 }
