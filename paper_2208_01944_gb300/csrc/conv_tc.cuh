@@ -303,14 +303,11 @@ __device__ __forceinline__ void producer_role(const ConvParams& p, const CUtenso
 // and each 16-byte chunk j of the K block's input channels there is a plane of
 // Hd x Wd positions (one 16-byte row per position); a position outside the image
 // is zero-filled (src-size 0), which is the zero padding.  Flat mode is one row
-// of flat_box positions.  The (position, chunk) pattern of a plane row is the same
-// for every row, so each thread precomputes its share once.  A thread releases a
-// stage after its copies have landed (wait_group) and a proxy fence, so the
+// of flat_box positions.  A thread releases a stage after its copies have landed (wait_group) and a proxy fence, so the
 // tensor core (async proxy) sees the data; up to `depth` newer stages per thread
 // stay in flight meanwhile.
 // --------------------------------------------------------------------------
 constexpr int kLoaders = 32 * kLoadWarps;
-constexpr int kMaxLoadEntries = 8;
 
 // Every thread's copies of the stage have landed (its wait_group); after the
 // proxy fence and a warp barrier one lane arrives for the warp.
@@ -325,40 +322,27 @@ __device__ __forceinline__ void loader_role(const ConvParams& p, const Bars& bar
   if (p.a_tma) return;  // warp 0 loads the operand with TMA
   const int tid = threadIdx.x - 32 * kFirstLoadWarp;
   const bool flat = p.mode == kModeFlat;
-  const int nch = p.nch;
+  const uint32_t nch = static_cast<uint32_t>(p.nch), nch_magic = p.nch_magic;
   const uint32_t plane = p.lbo_a;
-  const int64_t ld_pix = p.ld_pix, ld_chunk = p.ld_chunk;
-  const int row_len = flat ? p.flat_box : p.Wd;
-  const int per_row = row_len * nch;
-  const bool tabled = per_row <= kMaxLoadEntries * kLoaders;
-  // This thread's (position, chunk) entries of one plane row.
-  uint32_t ent_dst[kMaxLoadEntries];
-  int ent_iw0[kMaxLoadEntries], ent_jo[kMaxLoadEntries];  // ent_jo: the entry's 16-channel chunk
-  int n_ent = 0;
-#pragma unroll
-  for (int i = 0; i < kMaxLoadEntries; ++i) {
-    const int e = tid + i * kLoaders;
-    ent_dst[i] = 0;
-    ent_iw0[i] = 0;
-    ent_jo[i] = 0;
-    if (tabled && e < per_row) {
-      const int w = static_cast<int>(__umulhi(static_cast<uint32_t>(e), p.nch_magic));
-      const int j = e - w * nch;
-      ent_dst[i] = static_cast<uint32_t>(j) * plane + static_cast<uint32_t>(w) * 16u;
-      ent_iw0[i] = flat ? w : p.stride * (p.w_coord + w);
-      ent_jo[i] = j;
-      n_ent = i + 1;
-    }
-  }
-  // Per-row values that depend on the stride phase, held in registers (a
-  // dynamically indexed kernel-parameter array costs a long-latency load).
-  const int pa0 = p.phase_a[0], pa1 = p.phase_a[1], pa2 = p.phase_a[2], pa3 = p.phase_a[3];
-  const int pb0 = p.phase_b[0], pb1 = p.phase_b[1], pb2 = p.phase_b[2], pb3 = p.phase_b[3];
+  const int64_t ld_pix = p.ld_pix, ld_chunk = p.ld_chunk, ld_row = p.ld_row;
+  const uint32_t row_len = static_cast<uint32_t>(flat ? p.flat_box : p.Wd), per_row = row_len * nch;
+  const uint32_t row_magic = static_cast<uint32_t>(((1ull << 32) + per_row - 1) / per_row);
+  // The copies of a stage are a list of (plane row, position, chunk), the chunk fastest:
+  // a thread takes every 128th, a few divisions by multiplication each.  (Row by row,
+  // with the row's entries in a table of eight per thread, a stage of 960 copies took
+  // 8700 cycles to issue, mostly in predicated entries that no thread had: 20x37x45, 3
+  // groups of 96, NHWC, with its quantiser 47.3 us, now 43.0.)
   const int depth = min(2, p.a_stages - 1);
   Ring ra{0, 0, static_cast<uint32_t>(p.a_stages)};
   int64_t issued = 0, released = 0;
   bool ok = true;
   const int nph = flat ? 1 : p.nph, Hd = flat ? 1 : p.Hd;
+  const int stride = flat ? 1 : p.stride, w0 = flat ? 0 : p.w_coord;
+  // Per-phase values, held in registers (a dynamically indexed kernel-parameter array
+  // costs a long-latency load).
+  const int pa0 = p.phase_a[0], pa1 = p.phase_a[1], pa2 = p.phase_a[2], pa3 = p.phase_a[3];
+  const int pb0 = p.phase_b[0], pb1 = p.phase_b[1], pb2 = p.phase_b[2], pb3 = p.phase_b[3];
+  const uint32_t entries = static_cast<uint32_t>(Hd) * per_row;  // of one phase
   Item item = item_begin(p, it0);
   pin(item);
   if (p.pdl && !p.pdl_early_loads) wait_previous_grid();
@@ -367,48 +351,24 @@ __device__ __forceinline__ void loader_role(const ConvParams& p, const Bars& bar
       if (!warp_wait(bars.a_empty(ra.stage), ra.phase ^ 1u, ctx)) { ok = false; break; }
       const uint32_t stage = a_base + ra.stage * p.a_stage_bytes;
       const int ch0 = p.group[item.g].src * p.Cin_g + kb * p.KC;  // first input channel of the K block
-      const uint8_t* img_src = p.q_in + item.n * p.ld_img + static_cast<int64_t>(ch0) * p.ld_c0_mul / 16;
-      for (int ph = 0; ph < nph; ++ph)
-      for (int r = 0; r < Hd; ++r) {
-        bool row_ok;
-        const uint8_t* row_src;
-        uint32_t row_dst;
-        int b, w_lim;
-        if (flat) {
-          const int p0 = item.rb * p.flat_box;  // first pixel of the tile in its image
-          row_ok = true;
-          row_src = img_src + static_cast<int64_t>(p0) * ld_pix;
-          row_dst = stage;
-          b = 0;
-          w_lim = min(p.img_pix - p0, p.flat_box);
-        } else {
-          const int pa = ph == 0 ? pa0 : ph == 1 ? pa1 : ph == 2 ? pa2 : pa3;
-          const int ih = p.stride * (item.oh0(p.Ht) + p.h_off + r) + pa;
-          row_ok = ih >= 0 && ih < p.H;
-          row_src = img_src + (row_ok ? ih : 0) * p.ld_row;
-          row_dst = stage + ph * p.a_phase_bytes + static_cast<uint32_t>(r * p.Wd) * 16u;
-          b = ph == 0 ? pb0 : ph == 1 ? pb1 : ph == 2 ? pb2 : pb3;
-          w_lim = p.W;
-        }
-        if (tabled) {
-#pragma unroll
-          for (int i = 0; i < kMaxLoadEntries; ++i) {
-            if (i < n_ent) {
-              const int iw = ent_iw0[i] + b;
-              const bool valid = row_ok && iw >= 0 && iw < w_lim;
-              cp_async_16(row_dst + ent_dst[i], valid ? row_src + iw * ld_pix + ent_jo[i] * ld_chunk : p.q_in,
-                          valid ? 16u : 0u);
-            }
-          }
-        } else {
-          for (int e = tid; e < per_row; e += kLoaders) {
-            const int w = static_cast<int>(__umulhi(static_cast<uint32_t>(e), p.nch_magic));
-            const int j = e - w * nch;
-            const int iw = (flat ? w : p.stride * (p.w_coord + w)) + b;
-            const bool valid = row_ok && iw >= 0 && iw < w_lim;
-            cp_async_16(row_dst + static_cast<uint32_t>(j) * plane + static_cast<uint32_t>(w) * 16u,
-                        valid ? row_src + iw * ld_pix + j * ld_chunk : p.q_in, valid ? 16u : 0u);
-          }
+      const int p0 = flat ? item.rb * p.flat_box : 0;             // flat: first pixel of the tile in its image
+      const uint8_t* img_src = p.q_in + item.n * p.ld_img + static_cast<int64_t>(ch0) * p.ld_c0_mul / 16 +
+                               static_cast<int64_t>(p0) * ld_pix;
+      const int w_lim = flat ? min(p.img_pix - p0, p.flat_box) : p.W;
+      const int h0 = flat ? 0 : item.oh0(p.Ht) + p.h_off;
+      for (int ph = 0; ph < nph; ++ph) {
+        const int pa = flat ? 0 : (ph == 0 ? pa0 : ph == 1 ? pa1 : ph == 2 ? pa2 : pa3);
+        const int pb = flat ? 0 : (ph == 0 ? pb0 : ph == 1 ? pb1 : ph == 2 ? pb2 : pb3);
+        const uint32_t phase_dst = stage + ph * p.a_phase_bytes;
+        const int h_lim = flat ? 1 : p.H;
+#pragma unroll 4
+        for (uint32_t e = tid; e < entries; e += kLoaders) {
+          const uint32_t r = __umulhi(e, row_magic), in_row = e - r * per_row;
+          const uint32_t w = __umulhi(in_row, nch_magic), j = in_row - w * nch;
+          const int ih = stride * (h0 + static_cast<int>(r)) + pa, iw = stride * (w0 + static_cast<int>(w)) + pb;
+          const bool valid = ih >= 0 && ih < h_lim && iw >= 0 && iw < w_lim;
+          cp_async_16(phase_dst + j * plane + (r * row_len + w) * 16u,
+                      valid ? img_src + ih * ld_row + iw * ld_pix + j * ld_chunk : p.q_in, valid ? 16u : 0u);
         }
       }
       cp_async_commit();
