@@ -1293,6 +1293,15 @@ __device__ __forceinline__ void epilogue_role(const ConvParams& p, const Bars& b
     if (item.g != cur_g) load_group(item.g);
     if (!warp_wait(bars.acc_full(racc.stage), racc.phase, ctx)) break;
     tc_fence_after();
+    // One arrival per warp: the warp's tensor-memory reads are complete (each thread
+    // waited for its loads) and ordered before the arrive by the fence and the warp
+    // barrier.  The codes-only paths arrive before their last unit's conversion and store
+    // (128x28x28, 8 groups of 64, FP4 codes: 29.4 us, now 28.2).
+    auto release_acc = [&]() {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bars.acc_empty(racc.stage));
+    };
     EpiItem e;
     e.g = item.g;
     e.nb = item.nb;
@@ -1340,6 +1349,7 @@ __device__ __forceinline__ void epilogue_role(const ConvParams& p, const Bars& b
         tmem_ld16(col(c_mt, c_b) + 16, vb);
         const uint2 lo = pack4_word(epi_codes16_f16(va, e.m_req15, qmax2));
         tmem_wait_ld();
+        if (left == 1) release_acc();
         int n_mt = c_mt, n_b = c_b + 1;
         if (n_b == per_acc) {
           n_b = 0;
@@ -1400,6 +1410,7 @@ __device__ __forceinline__ void epilogue_role(const ConvParams& p, const Bars& b
         uint8_t* c_row = row_ptr(c_mt);
         uint8_t* n_row = two ? (n_mt == c_mt ? c_row : row_ptr(n_mt)) : nullptr;
         tmem_wait_ld();
+        if (left <= 2) release_acc();
         const uint4 w0 = epi_codes16_f16(va, e.m_req15, qmax2);
         const uint4 w1 = epi_codes16_f16(vb, e.m_req15, qmax2);
         if (c_row) store_codes16(c_row + coff(c_ch), w0, pack);
@@ -1409,12 +1420,7 @@ __device__ __forceinline__ void epilogue_role(const ConvParams& p, const Bars& b
         c_ch = n_ch;
       }
     }
-    // One arrival per warp: the warp's tensor-memory reads are complete (each
-    // thread waited for its loads) and ordered before the arrive by the fence
-    // and the warp barrier.
-    tc_fence_before();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(bars.acc_empty(racc.stage));
+    if (GEN || u_count == 0) release_acc();
     racc.advance();
   }
   if constexpr (GEN) cp_async_wait<0>();  // after an abort, the rows fetched ahead
