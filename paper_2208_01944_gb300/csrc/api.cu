@@ -469,7 +469,6 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub,
                              16ull * (p.MT * 128 + off_max);
     return round_up(std::max<uint64_t>(static_cast<uint64_t>(p.nph) * (*phase_bytes), overrun), 1024);
   };
-  const uint32_t q_pitch = 80;
   // Staging for every warp that runs the epilogue: the copy warps join it only when
   // TMA loads the activation operand as it is (not unpacked, not quantised).
   const bool third_group =
@@ -627,7 +626,6 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub,
   p.smem_pk_off = p.smem_stage_off + stage_total;  // packed staging ring (a_stages x pk_stage_bytes)
   p.smem_bar_off = p.smem_pk_off + static_cast<uint32_t>(a_stages) * p.pk_stage_bytes;
   p.smem_bytes = p.smem_bar_off + bar_bytes;
-  p.stage_q_pitch = q_pitch;
   p.stage_warp_bytes = warp_stage;
   p.C_out_total = d->G * d->Cout_g;
   p.relu = d->relu;

@@ -714,22 +714,6 @@ __device__ __forceinline__ void mma_role_dispatch(const ConvParams& p, const Bar
 // --------------------------------------------------------------------------
 // Epilogue role (warps 2-5).
 // --------------------------------------------------------------------------
-// 32 rows of `row_bytes` (multiple of 16) staged at `pitch`: lane r's row goes to
-// global byte offset row_off (negative: row not stored).
-__device__ __forceinline__ void warp_store_rows(const uint8_t* stg, uint32_t pitch, int row_bytes, uint8_t* gdst,
-                                                long long row_off, int lane) {
-  __syncwarp();
-  const int cpr = row_bytes >> 4;
-  const int total = 32 * cpr;
-  for (int idx = lane; idx < total; idx += 32) {
-    const int r = idx / cpr;
-    const int c = idx - r * cpr;
-    const long long off = __shfl_sync(0xffffffffu, row_off, r);
-    if (off >= 0) *reinterpret_cast<uint4*>(gdst + off + c * 16) = *reinterpret_cast<const uint4*>(stg + r * pitch + c * 16);
-  }
-  __syncwarp();
-}
-
 // Requantised code of t = clamp(rint(t), 0, qmax) with round-half-to-even, on the
 // FMA and integer pipes: clamping t to [-1, qmax + 1] first does not change the
 // result (rounding is monotone and the final clamp is integral), and for
@@ -832,14 +816,6 @@ __device__ __forceinline__ void store_codes16(uint8_t* dst, uint4 w, int pack) {
     *reinterpret_cast<uint2*>(dst) = pack4_word(w);
   else
     *reinterpret_cast<uint4*>(dst) = w;
-}
-
-// Byte offset of the 16 codes of output pixel pos (in its image n) and the
-// 16-channel chunk k = channel / 16, channel-blocked.
-__device__ __forceinline__ long long codes_offset(const ConvParams& p, int pack, int n, long long hw_out, int pos, int k) {
-  if (pack == 2)
-    return ((static_cast<long long>(n) * (p.C_out_total >> 5) + (k >> 1)) * hw_out + pos) * 16 + (k & 1) * 8;
-  return ((static_cast<long long>(n) * (p.C_out_total >> 4) + k) * hw_out + pos) * (pack ? 4 : 16);
 }
 
 // --------------------------------------------------------------------------
@@ -947,48 +923,36 @@ __device__ __forceinline__ void quant_role(const ConvParams& p, const Bars& bars
   }
 }
 
-// Store 16 codes of 16-column chunk `ch` of this lane's row.
-__device__ __forceinline__ void epi_store_codes(const ConvParams& p, const EpiItem& e, uint8_t* stg, int lane, uint32_t row,
-                                                int ch, uint4 w) {
-  const long long hw_out = static_cast<long long>(p.Ho) * p.Wo;
-  const bool valid = row_valid(e, row);
-  const int n = e.n + row_img(row), pos = e.pos0 + row_pos(row);
-  if (p.codes_c16) {
-    // Channel-blocked codes: lanes hold consecutive pixels, so each store of the
-    // warp lands next to its neighbours'.
-    if (valid) {
-      const int pack = codes_pack(p);
-      store_codes16(p.q_out + codes_offset(p, pack, n, hw_out, pos, (e.dst_c0 >> 4) + ch), w, pack);
-    }
-  } else {
-    // NHWC: staged, then 16-byte rows written by the warp.
-    *reinterpret_cast<uint4*>(stg + lane * p.stage_q_pitch) = w;
-    const long long pix = static_cast<long long>(n) * hw_out + pos;
-    warp_store_rows(stg, p.stage_q_pitch, 16, p.q_out, valid ? pix * p.C_out_total + e.dst_c0 + ch * 16 : -1, lane);
-  }
+// General units (int32 sums, fp32 outputs with or without the shortcut, codes) of UC
+// accumulator columns.  TMEM gives each lane one row (pixel), but a global access
+// instruction costs about one cycle per cache line it touches, so rows of 4 UC bytes per
+// lane would cost 32 lines per instruction.  The shortcut, the fp32 outputs and the int32
+// sums therefore pass through the warp's staging buffer (32 rows of 4 UC bytes; 16-byte
+// chunk c of row r at chunk c ^ sw(r), which keeps both access patterns conflict-free): a
+// global access instruction takes whole rows, 512 bytes in 4 rows of 128 (UC = 32) or 8
+// rows of 64 (UC = 16), and each lane reads or writes its own row in shared memory.  The
+// shortcut comes by cp.async (zero-filled for rows outside the output).  Codes go through
+// the fp16 conversion (epi_codes16_f16) where no NaN can reach it: without a shortcut the
+// value is fl(raw * m_req * 2^-15) = fl(acc * m_req) * 2^-24; with one,
+// fl(y * m_req * 2^-24) = fl(y * m_req) * 2^-24 (a power-of-two factor, exact while the
+// product is normal; both give code 0 below that), and ReLU has removed NaN
+// (fmaxf(NaN, 0) = 0).  A shortcut without ReLU keeps the scalar form, which maps NaN to
+// code 0.
+//
+// Instruction fetch bounds these units before memory does (the largest stall of the
+// 128x56x56 layer with shortcut when a unit took 900 instructions), so addresses are a
+// 64-bit base per item plus a 32-bit pixel times the row's bytes, a row's entry is
+// computed when the accumulator changes, and units advance without divisions.
+template <int UC>
+__device__ __forceinline__ uint32_t row_swizzle(int r) {
+  constexpr int CPR = UC / 4;  // 16-byte chunks per staged row
+  return static_cast<uint32_t>((UC == 32 ? r : r >> 1) & (CPR - 1)) << 4;
 }
 
-// General units (int32 sums, fp32 outputs with or without the shortcut, codes)
-// of UC accumulator columns.  TMEM gives each lane one row (pixel), but a global
-// access instruction costs about one cycle per cache line it touches, so rows
-// of 4 UC bytes per lane would cost 32 lines per instruction.  The shortcut,
-// the fp32 outputs and the int32 sums therefore pass through the warp's staging
-// buffer (32 rows of 4 UC bytes; 16-byte chunk c of row r at chunk c ^ sw(r),
-// which keeps both access patterns conflict-free): a global access instruction
-// takes whole rows, 512 bytes in 4 rows of 128 (UC = 32) or 8 rows of 64
-// (UC = 16), and each lane reads or writes its own row in shared memory.  The shortcut comes by
-// cp.async (zero-filled for rows outside the output).  Codes go through the
-// fp16 conversion (epi_codes16_f16) where no NaN can reach it: without a
-// shortcut the value is fl(raw * m_req * 2^-15) = fl(acc * m_req) * 2^-24; with
-// one, fl(y * m_req * 2^-24) = fl(y * m_req) * 2^-24 (a power-of-two factor,
-// exact while the product is normal; both give code 0 below that), and ReLU has
-// removed NaN (fmaxf(NaN, 0) = 0).  A shortcut without ReLU keeps the scalar
-// form, which maps NaN to code 0.
-template <int UC>
-__device__ __forceinline__ uint32_t stg_chunk(uint32_t base, int r, int c) {
-  constexpr int CPR = UC / 4;  // 16-byte chunks per staged row
-  const int sw = (UC == 32 ? r : r >> 1) & (CPR - 1);
-  return base + static_cast<uint32_t>(r * (UC * 4) + ((c ^ sw) << 4));
+// A lane's pixel in its tile's item, from the item's first pixel on (-1: none).
+__device__ __forceinline__ int row_pixel(const ConvParams& p, int m, int bound) {
+  const uint32_t row = row_entry(p, m);
+  return static_cast<int>(row >> 19) < bound ? row_img(row) * p.Ho * p.Wo + row_pos(row) : -1;
 }
 
 // Where an item's rows lie in the output (and in the shortcut).
@@ -1007,40 +971,40 @@ __device__ __forceinline__ RowSpan row_span(const ConvParams& p, const Item& ite
   return r;
 }
 
-// Unit u's shortcut rows (its source channels) into the staging buffer `buf` by
-// cp.async, whole rows per instruction, zero-filled outside the output.
+// Element offset of channel c0 of an item's first pixel in an NHWC output.
+__device__ __forceinline__ long long span_offset(const ConvParams& p, int n, int pos0, int c0) {
+  return (static_cast<long long>(n) * p.Ho * p.Wo + pos0) * p.C_out_total + c0;
+}
+
+// A unit's shortcut rows (UC columns from `src` on: the item's first pixel, the unit's
+// first channel) into the staging buffer `buf` by cp.async, whole rows per instruction,
+// zero-filled outside the output; `pix` is this lane's pixel.
 template <int UC>
-__device__ __forceinline__ void fetch_shortcut(const ConvParams& p, const RowSpan& sp, int u, int m_lane, int lane,
-                                               uint32_t buf) {
+__device__ __forceinline__ void fetch_shortcut(const ConvParams& p, const float* src, int pix, int lane, uint32_t buf) {
   constexpr int CPR = UC / 4, RPP = 32 / CPR;  // chunks per row, rows per coalesced pass
-  const int per_acc = p.Nblk / UC, mt = u / per_acc, col0 = (u - mt * per_acc) * UC;
-  const uint32_t row = row_entry(p, mt * 128 + m_lane);
-  const long long hw_out = static_cast<long long>(p.Ho) * p.Wo;
-  const long long rc =
-      static_cast<int>(row >> 19) < sp.bound
-          ? ((sp.n + row_img(row)) * hw_out + sp.pos0 + row_pos(row)) * p.C_out_total
-          : -1;
   const int pr = lane / CPR, pc = lane % CPR;  // row within a pass, chunk: coalesced role
-  const float* const src = p.shortcut + sp.src_c0 + col0 + 4 * pc;
+  const uint32_t row_bytes = 4u * static_cast<uint32_t>(p.C_out_total);
+  const uint8_t* const s0 = reinterpret_cast<const uint8_t*>(src + 4 * pc);
 #pragma unroll
   for (int ps = 0; ps < CPR; ++ps) {
     const int r = ps * RPP + pr;
-    const long long off = __shfl_sync(0xffffffffu, rc, r);
-    cp_async_16(stg_chunk<UC>(buf, r, pc), off >= 0 ? src + off : p.shortcut, off >= 0 ? 16u : 0u);
+    const int px = __shfl_sync(0xffffffffu, pix, r);
+    cp_async_16(buf + static_cast<uint32_t>(r * (UC * 4)) + ((static_cast<uint32_t>(pc) << 4) ^ row_swizzle<UC>(r)),
+                s0 + static_cast<uint64_t>(static_cast<uint32_t>(max(px, 0))) * row_bytes, px >= 0 ? 16u : 0u);
   }
   cp_async_commit();
 }
 
 // `cur`: the staging buffer that holds the unit's shortcut rows (fetched ahead); `item`
 // the item and `more` whether this CTA has another one.
-template <int UC>
+template <int UC, bool F4>
 __device__ __forceinline__ void epi_general_units(const ConvParams& p, const EpiItem& e, uint8_t* stg, int wg,
                                                   int n_groups, int m_lane, int lane, uint32_t qmax2, const Item& item,
                                                   bool more, int& cur) {
   constexpr int CPR = UC / 4, RPP = 32 / CPR;  // chunks per row, rows per coalesced pass
-  // one staging buffer: 32 rows of 128 bytes whatever UC is, so that the NHWC code
-  // rows staged by epi_store_codes (32 rows at an 80-byte pitch) stay inside it
-  constexpr uint32_t kBuf = 32u * 128u;
+  // one staging buffer: 32 rows of 128 bytes whatever UC is, so that NHWC code rows
+  // (32 rows at an 80-byte pitch) stay inside it
+  constexpr uint32_t kBuf = 32u * 128u, kCodePitch = 80u;
   const bool has_sc = p.shortcut != nullptr;
   // With a shortcut (and no int32 output, which would need the buffer first) the
   // next unit's shortcut rows, also across items, are fetched into the warp's second
@@ -1050,42 +1014,55 @@ __device__ __forceinline__ void epi_general_units(const ConvParams& p, const Epi
   const bool pre = has_sc && p.acc_out == nullptr;
   const bool f16q = !has_sc || p.relu;
   const float m_q = has_sc ? __fmul_rn(e.m_req, 1.0f / 16777216.0f) : e.m_req15;
-  const int qmax = p.qmax_out;
-  const float qmax_f = static_cast<float>(qmax);
-  const long long hw_out = static_cast<long long>(p.Ho) * p.Wo;
   const int per_acc = p.Nblk / UC;
-  // The warpgroups take the units in turn, so that the column chunks of a row are
-  // read and written at about the same time (as contiguous runs per warpgroup, 128x56x56
-  // with shortcut, fp32 and codes out took 116 us against 100).
-  const int n_units = p.MT * per_acc;
+  const uint32_t row_bytes = 4u * static_cast<uint32_t>(p.C_out_total);
+  const long long dst0 = span_offset(p, e.n, e.pos0, e.dst_c0);
+  const float* const sc0 = p.shortcut + span_offset(p, e.n, e.pos0, e.src_c0);
   const int pr = lane / CPR, pc = lane % CPR;  // row within a pass, chunk: coalesced role
   // Channel shuffle (kind 2): column j of the unit goes to destination channel
   // (nb Nblk + col0 + j) G + g, so a staged row leaves as UC values G apart:
   // lane j of a store instruction takes column j of 32 / UC rows.
   const bool shuf = p.channel_shuffle != 0;
-  const int sj = lane % UC, sr = lane / UC;
-  // this lane's row of unit u, and its offset (elements; -1 outside the output)
-  const long long row0 = static_cast<long long>(e.n) * hw_out + e.pos0;
-  auto row_off = [&](uint32_t r) -> long long {
-    return row_valid(e, r) ? (row0 + row_img(r) * static_cast<int>(hw_out) + row_pos(r)) * p.C_out_total : -1;
-  };
-  auto row_at = [&](int u) { return row_entry(p, u / per_acc * 128 + m_lane); };
-  for (int u = wg; u < n_units; u += n_groups, cur ^= 1) {
-    const int mt = u / per_acc, col0 = (u - mt * per_acc) * UC;
-    const uint32_t row = row_at(u);
-    const long long rowc = row_off(row);
+  // The warpgroups take the units in turn, so that the column chunks of a row are
+  // read and written at about the same time (as contiguous runs per warpgroup, 128x56x56
+  // with shortcut, fp32 and codes out took 116 us against 100).
+  int mt = 0, b = wg;  // the unit: accumulator and column chunk
+  while (b >= per_acc) {
+    b -= per_acc;
+    ++mt;
+  }
+  int pix = row_pixel(p, mt * 128 + m_lane, e.bound);
+  while (mt < p.MT) {
+    const int col0 = b * UC;
+    // the unit after this one
+    int n_mt = mt, n_b = b + n_groups;
+    while (n_b >= per_acc) {
+      n_b -= per_acc;
+      ++n_mt;
+    }
+    int n_pix = pix;
+    if (n_mt != mt && n_mt < p.MT) n_pix = row_pixel(p, n_mt * 128 + m_lane, e.bound);
     const uint32_t sbase = smem_u32(stg) + (pre ? static_cast<uint32_t>(cur) * kBuf : 0u);
-    uint8_t* const stg_cur = stg + (pre ? cur * kBuf : 0u);
     if (pre) {
-      const uint32_t next_buf = smem_u32(stg) + static_cast<uint32_t>(cur ^ 1) * kBuf;
-      if (u + n_groups < n_units) {
-        fetch_shortcut<UC>(p, RowSpan{e.n, e.pos0, e.bound, e.src_c0}, u + n_groups, m_lane, lane, next_buf);
-        cp_async_wait<1>();  // this unit's rows have landed; the next unit's may still be in flight
-      } else if (more) {
+      const float* n_src = sc0 + n_b * UC;
+      int f_pix = n_pix;
+      bool fetch = n_mt < p.MT;
+      if (!fetch && more) {
         Item next = item;
         item_next(p, next);
-        fetch_shortcut<UC>(p, row_span(p, next), wg, m_lane, lane, next_buf);
-        cp_async_wait<1>();
+        const RowSpan sp = row_span(p, next);
+        int f_mt = 0, f_b = wg;
+        while (f_b >= per_acc) {
+          f_b -= per_acc;
+          ++f_mt;
+        }
+        n_src = p.shortcut + span_offset(p, sp.n, sp.pos0, sp.src_c0) + f_b * UC;
+        f_pix = row_pixel(p, f_mt * 128 + m_lane, sp.bound);
+        fetch = true;
+      }
+      if (fetch) {
+        fetch_shortcut<UC>(p, n_src, f_pix, lane, smem_u32(stg) + static_cast<uint32_t>(cur ^ 1) * kBuf);
+        cp_async_wait<1>();  // this unit's rows have landed; the next unit's may still be in flight
       } else {
         cp_async_wait<0>();
       }
@@ -1096,33 +1073,43 @@ __device__ __forceinline__ void epi_general_units(const ConvParams& p, const Epi
       tmem_ld32(e.tbase + mt * p.Npow2 + col0, v);
     else
       tmem_ld16(e.tbase + mt * p.Npow2 + col0, v);
-    // Whole staged rows to global memory (row r's element offset is lane r's rowc).
-    auto store_rows = [&](void* out, int c0) {
+    // this lane's row in the staging buffer: chunk c at own ^ (c << 4)
+    const uint32_t own = sbase + static_cast<uint32_t>(lane * (UC * 4)) + row_swizzle<UC>(lane);
+    // Whole staged rows to global memory, from channel c0 of the item's first pixel on.
+    auto store_rows = [&](void* out) {
       __syncwarp();
       if (shuf) {
-        const long long dcl = static_cast<long long>(e.nb * p.Nblk + col0 + sj) * p.G + e.g;
+        const int sj = lane % UC, sr = lane / UC;
+        uint32_t* const o = reinterpret_cast<uint32_t*>(out) + span_offset(p, e.n, e.pos0, 0) +
+                            static_cast<long long>(e.nb * p.Nblk + col0 + sj) * p.G + e.g;
 #pragma unroll 4
         for (int r0 = 0; r0 < 32; r0 += 32 / UC) {
           const int r = r0 + sr;
-          const long long off = __shfl_sync(0xffffffffu, rowc, r);
+          const int px = __shfl_sync(0xffffffffu, pix, r);
           uint32_t x;
-          asm volatile("ld.shared.b32 %0, [%1];" : "=r"(x) : "r"(stg_chunk<UC>(sbase, r, sj >> 2) + 4u * (sj & 3)) : "memory");
-          if (off >= 0) reinterpret_cast<uint32_t*>(out)[off + dcl] = x;
+          asm volatile("ld.shared.b32 %0, [%1];"
+                       : "=r"(x)
+                       : "r"(sbase + static_cast<uint32_t>(r * (UC * 4)) +
+                             ((static_cast<uint32_t>(sj >> 2) << 4) ^ row_swizzle<UC>(r)) + 4u * (sj & 3))
+                       : "memory");
+          if (px >= 0) o[static_cast<long long>(px) * p.C_out_total] = x;
         }
         __syncwarp();
         return;
       }
+      uint8_t* const o = reinterpret_cast<uint8_t*>(out) + 4 * (dst0 + col0 + 4 * pc);
 #pragma unroll
       for (int ps = 0; ps < CPR; ++ps) {
         const int r = ps * RPP + pr;
-        const long long off = __shfl_sync(0xffffffffu, rowc, r);
+        const int px = __shfl_sync(0xffffffffu, pix, r);
         uint32_t x0, x1, x2, x3;
         asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
                      : "=r"(x0), "=r"(x1), "=r"(x2), "=r"(x3)
-                     : "r"(stg_chunk<UC>(sbase, r, pc))
+                     : "r"(sbase + static_cast<uint32_t>(r * (UC * 4)) +
+                           ((static_cast<uint32_t>(pc) << 4) ^ row_swizzle<UC>(r)))
                      : "memory");
-        if (off >= 0)
-          *reinterpret_cast<uint4*>(reinterpret_cast<uint32_t*>(out) + off + c0 + col0 + 4 * pc) =
+        if (px >= 0)
+          *reinterpret_cast<uint4*>(o + static_cast<uint64_t>(static_cast<uint32_t>(px)) * row_bytes) =
               make_uint4(x0, x1, x2, x3);
       }
       __syncwarp();
@@ -1131,7 +1118,7 @@ __device__ __forceinline__ void epi_general_units(const ConvParams& p, const Epi
     auto stage_row = [&](const uint32_t (&x)[UC]) {
 #pragma unroll
       for (int c = 0; c < CPR; ++c)
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stg_chunk<UC>(sbase, lane, c)), "r"(x[4 * c]),
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(own ^ static_cast<uint32_t>(c << 4)), "r"(x[4 * c]),
                      "r"(x[4 * c + 1]), "r"(x[4 * c + 2]), "r"(x[4 * c + 3])
                      : "memory");
     };
@@ -1142,11 +1129,11 @@ __device__ __forceinline__ void epi_general_units(const ConvParams& p, const Epi
       for (int j = 0; j < UC; ++j) a[j] = static_cast<uint32_t>(__float2int_rn(__fmul_rn(__uint_as_float(v[j]), 512.0f)));
       __syncwarp();
       stage_row(a);
-      store_rows(p.acc_out, e.dst_c0);
+      store_rows(p.acc_out);
     }
     if (has_sc && !pre) {
       // the rows' shortcut values into the staging buffer, after the int32 sums left it
-      fetch_shortcut<UC>(p, RowSpan{e.n, e.pos0, e.bound, e.src_c0}, u, m_lane, lane, sbase);
+      fetch_shortcut<UC>(p, sc0 + col0, pix, lane, sbase);
       cp_async_wait<0>();
       __syncwarp();
     }
@@ -1158,27 +1145,33 @@ __device__ __forceinline__ void epi_general_units(const ConvParams& p, const Epi
     }
     // y = relu(fl(acc * m_out) + shortcut), in place
 #pragma unroll
-    for (int c = 0; c < CPR; ++c) {
-      float sc0 = 0.0f, sc1 = 0.0f, sc2 = 0.0f, sc3 = 0.0f;
-      if (has_sc)
-        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                     : "=f"(sc0), "=f"(sc1), "=f"(sc2), "=f"(sc3)
-                     : "r"(stg_chunk<UC>(sbase, lane, c))
-                     : "memory");
-      const float scv[4] = {sc0, sc1, sc2, sc3};
+    for (int j = 0; j < UC; ++j)
+      v[j] = __float_as_uint(__fmul_rn(__uint_as_float(v[j]), e.m_out512));  // = (float)acc * m_out, one rounding
+    if (has_sc) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        float t = __fmul_rn(__uint_as_float(v[4 * c + k]), e.m_out512);  // = (float)acc * m_out, one rounding
-        if (has_sc) t = __fadd_rn(t, scv[k]);
-        if (p.relu) t = fmaxf(t, 0.0f);
-        v[4 * c + k] = __float_as_uint(t);
+      for (int c = 0; c < CPR; ++c) {
+        float s0, s1, s2, s3;
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                     : "=f"(s0), "=f"(s1), "=f"(s2), "=f"(s3)
+                     : "r"(own ^ static_cast<uint32_t>(c << 4))
+                     : "memory");
+        v[4 * c] = __float_as_uint(__fadd_rn(__uint_as_float(v[4 * c]), s0));
+        v[4 * c + 1] = __float_as_uint(__fadd_rn(__uint_as_float(v[4 * c + 1]), s1));
+        v[4 * c + 2] = __float_as_uint(__fadd_rn(__uint_as_float(v[4 * c + 2]), s2));
+        v[4 * c + 3] = __float_as_uint(__fadd_rn(__uint_as_float(v[4 * c + 3]), s3));
       }
+    }
+    if (p.relu) {
+#pragma unroll
+      for (int j = 0; j < UC; ++j) v[j] = __float_as_uint(fmaxf(__uint_as_float(v[j]), 0.0f));
     }
     if (p.q_out && has_sc) {
       if (f16q) {
         w[0] = epi_codes16_f16<UC, 0>(v, m_q, qmax2);
         if constexpr (UC == 32) w[1] = epi_codes16_f16<UC, 16>(v, m_q, qmax2);
       } else {
+        const int qmax = p.qmax_out;
+        const float qmax_f = static_cast<float>(qmax);
 #pragma unroll
         for (int h = 0; h < UC / 16; ++h) {
           int code[16];
@@ -1195,26 +1188,90 @@ __device__ __forceinline__ void epi_general_units(const ConvParams& p, const Epi
     if (p.y_out) {
       __syncwarp();  // every lane has read its shortcut row
       stage_row(v);
-      store_rows(p.y_out, e.dst_c0);
+      store_rows(p.y_out);
     }
-    if (p.q_out && !shuf) {
-      __syncwarp();
+    if (p.q_out) {
+      // this lane's image and pixel in it
+      const int hw = p.Ho * p.Wo;
+      int img = 0, pos = pix;
+      if (p.ipt > 1 && pix > 0) {
+        img = pix / hw;
+        pos = pix - img * hw;
+      }
+      const long long hw_out = static_cast<long long>(p.Ho) * p.Wo;
+      if (shuf) {
+        if (pix >= 0) {
+          // byte codes scattered one by one (the API takes no packed codes here)
 #pragma unroll
-      for (int h = 0; h < UC / 16; ++h) epi_store_codes(p, e, stg_cur, lane, row, col0 / 16 + h, w[h]);
-    } else if (p.q_out && rowc >= 0) {
-      // byte codes scattered one by one (the API takes no packed codes here)
-#pragma unroll
-      for (int h = 0; h < UC / 16; ++h) {
-        const uint32_t wd[4] = {w[h].x, w[h].y, w[h].z, w[h].w};
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const long long dc = static_cast<long long>(e.nb * p.Nblk + col0 + 16 * h + j) * p.G + e.g;
-          const long long o = p.codes_c16 ? ((static_cast<long long>(e.n + row_img(row)) * (p.C_out_total >> 4) + (dc >> 4)) * hw_out + e.pos0 + row_pos(row)) * 16 + (dc & 15)
-                                          : rowc + dc;
-          p.q_out[o] = static_cast<uint8_t>(wd[j >> 2] >> (8 * (j & 3)));
+          for (int h = 0; h < UC / 16; ++h) {
+            const uint32_t wd[4] = {w[h].x, w[h].y, w[h].z, w[h].w};
+#pragma unroll 4
+            for (int j = 0; j < 16; ++j) {
+              const long long dc = static_cast<long long>(e.nb * p.Nblk + col0 + 16 * h + j) * p.G + e.g;
+              const long long o =
+                  p.codes_c16 ? ((static_cast<long long>(e.n + img) * (p.C_out_total >> 4) + (dc >> 4)) * hw_out + e.pos0 + pos) * 16 + (dc & 15)
+                              : span_offset(p, e.n, e.pos0, 0) + static_cast<long long>(pix) * p.C_out_total + dc;
+              p.q_out[o] = static_cast<uint8_t>(wd[j >> 2] >> (8 * (j & 3)));
+            }
+          }
         }
+      } else if (p.codes_c16) {
+        // Channel-blocked codes: lanes hold consecutive pixels, so each store of the
+        // warp lands next to its neighbours'.
+        if (pix >= 0) {
+          if (F4 && UC == 32) {
+            // the row of a 32-channel block (dst_c0 and the unit's columns are multiples of 32)
+            const uint2 lo = pack4_word(w[0]), hi = pack4_word(w[UC / 16 - 1]);
+            *reinterpret_cast<uint4*>(p.q_out + ((static_cast<long long>(e.n + img) * (p.C_out_total >> 5) + ((e.dst_c0 + col0) >> 5)) *
+                                                     hw_out + e.pos0 + pos) * 16) = make_uint4(lo.x, lo.y, hi.x, hi.y);
+          } else if (F4) {
+            const int k = (e.dst_c0 + col0) >> 4;
+            *reinterpret_cast<uint2*>(p.q_out + ((static_cast<long long>(e.n + img) * (p.C_out_total >> 5) + (k >> 1)) * hw_out +
+                                                 e.pos0 + pos) * 16 + (k & 1) * 8) = pack4_word(w[0]);
+          } else {
+            const int cb = p.codes_p2 ? 4 : 16;
+            uint8_t* o = p.q_out + ((static_cast<long long>(e.n + img) * (p.C_out_total >> 4) + ((e.dst_c0 + col0) >> 4)) * hw_out +
+                                    e.pos0 + pos) * cb;
+#pragma unroll
+            for (int h = 0; h < UC / 16; ++h, o += hw_out * cb) {
+              if (p.codes_p2)
+                *reinterpret_cast<uint32_t*>(o) = pack2_word(w[h]);
+              else
+                *reinterpret_cast<uint4*>(o) = w[h];
+            }
+          }
+        }
+      } else {
+        // NHWC: rows of UC bytes staged, then written by the warp in 16-byte pieces.
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < UC / 16; ++h)
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(sbase + static_cast<uint32_t>(lane) * kCodePitch + 16u * h),
+                       "r"(w[h].x), "r"(w[h].y), "r"(w[h].z), "r"(w[h].w)
+                       : "memory");
+        __syncwarp();
+        constexpr int PPR = UC / 16;  // pieces per row
+        uint8_t* const o = p.q_out + dst0 + col0 + 16 * (lane % PPR);
+#pragma unroll
+        for (int h = 0; h < PPR; ++h) {
+          const int r = h * (32 / PPR) + lane / PPR;
+          const int px = __shfl_sync(0xffffffffu, pix, r);
+          uint32_t x0, x1, x2, x3;
+          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                       : "=r"(x0), "=r"(x1), "=r"(x2), "=r"(x3)
+                       : "r"(sbase + static_cast<uint32_t>(r) * kCodePitch + 16u * (lane % PPR))
+                       : "memory");
+          if (px >= 0)
+            *reinterpret_cast<uint4*>(o + static_cast<uint64_t>(static_cast<uint32_t>(px)) * static_cast<uint32_t>(p.C_out_total)) =
+                make_uint4(x0, x1, x2, x3);
+        }
+        __syncwarp();
       }
     }
+    mt = n_mt;
+    b = n_b;
+    pix = n_pix;
+    cur ^= 1;
   }
 }
 
@@ -1283,10 +1340,13 @@ __device__ __forceinline__ void epilogue_role(const ConvParams& p, const Bars& b
     const int uc = (p.Nblk & 31) == 0 ? 32 : 16;
     if (p.shortcut != nullptr && p.acc_out == nullptr && wg < p.MT * (p.Nblk / uc)) {
       const RowSpan sp = row_span(p, item);
+      const int per = p.Nblk / uc, mt = wg / per, col0 = (wg - mt * per) * uc;
+      const float* src = p.shortcut + span_offset(p, sp.n, sp.pos0, sp.src_c0) + col0;
+      const int pix = row_pixel(p, mt * 128 + quarter * 32 + lane, sp.bound);
       if (uc == 32)
-        fetch_shortcut<32>(p, sp, wg, quarter * 32 + lane, lane, smem_u32(stg));
+        fetch_shortcut<32>(p, src, pix, lane, smem_u32(stg));
       else
-        fetch_shortcut<16>(p, sp, wg, quarter * 32 + lane, lane, smem_u32(stg));
+        fetch_shortcut<16>(p, src, pix, lane, smem_u32(stg));
     }
   }
   for (int64_t it = it0; it < it1; ++it, item_next(p, item)) {
@@ -1317,9 +1377,9 @@ __device__ __forceinline__ void epilogue_role(const ConvParams& p, const Bars& b
     e.tbase = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + racc.stage * p.MT * p.Npow2;
     if constexpr (GEN) {
       if ((p.Nblk & 31) == 0)
-        epi_general_units<32>(p, e, stg, wg, n_groups, quarter * 32 + lane, lane, qmax2, item, it + 1 < it1, cur);
+        epi_general_units<32, F4>(p, e, stg, wg, n_groups, quarter * 32 + lane, lane, qmax2, item, it + 1 < it1, cur);
       else
-        epi_general_units<16>(p, e, stg, wg, n_groups, quarter * 32 + lane, lane, qmax2, item, it + 1 < it1, cur);
+        epi_general_units<16, F4>(p, e, stg, wg, n_groups, quarter * 32 + lane, lane, qmax2, item, it + 1 < it1, cur);
     } else if (F4 && (p.Nblk & 31) == 0) {
       // FP4 nibbles, units of 32 columns: a lane's 32 codes are one whole 16-byte
       // row of a 32-channel block, so a unit costs one store instruction (the

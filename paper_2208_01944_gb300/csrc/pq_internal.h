@@ -135,7 +135,7 @@ struct ConvParams {
   // 1: 2-bit codes as packed FP4 (E2M1) nibbles, [N][C/32][H][W][16 B], read by the
   // block-scaled FP4 MMA; one 16-byte chunk then holds 32 channels.
   int codes_f4;
-  uint32_t stage_q_pitch, stage_warp_bytes;
+  uint32_t stage_warp_bytes;
   // ---- failure detection
   unsigned int* err;
   uint64_t wait_limit_ns;
