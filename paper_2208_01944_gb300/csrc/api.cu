@@ -509,7 +509,7 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub,
   // slices (the stage-4 conv1 of the network: 84 -> 72 us with conv1 + down once
   // its 147 KB of weights stayed at half the K block).
   bool found = false, resident = false;
-  int KC = d->Cin_g, a_stages = 0, b_stages = 0;
+  int KC = d->Cin_g, a_stages = 0, b_stages = 0, b_taps = 1;
   uint32_t stage_bytes = 0, phase_bytes = 0, lbo = 0;
   // K blocks of {8, 4, 3, 2, 1} MMA K steps (32 channels each, 64 for FP4): the
   // MMA issue loop is compiled for these K-step counts.
@@ -527,18 +527,26 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub,
       if (res && unit_bytes > 160u * 1024u) continue;
       const uint64_t slice = static_cast<uint64_t>(kc) * p.Nblk / cpb;
       if (!res && slice > 32u * 1024u) continue;
-      for (int na = 4; na >= 2 && !found; --na) {
-        for (int nb = (res ? 1 : 4); nb >= (res ? 1 : 2) && !found; --nb) {
-          const uint64_t bb = res ? round_up(unit_bytes, 1024) : round_up(nb * slice, 1024);
-          if (bb + stage_total + bar_bytes + static_cast<uint64_t>(na) * (sb + pk_stage_bytes(kc)) <= budget) {
-            found = true;
-            resident = res != 0;
-            KC = kc;
-            a_stages = na;
-            b_stages = nb;
-            stage_bytes = sb;
-            phase_bytes = pb;
-            lbo = l;
+      // Streamed weights: as many taps to a ring stage as 32 KB hold, then one.  A stage
+      // costs a round of barriers, and with one small slice each (channel counts whose
+      // largest K block is 32) those set the pace: 2x19x17, 4 groups of 224, codes, 23.1 ->
+      // 17.8 us (128x28x28, 2 groups of 256, whose slices are 32 KB, 81.7 -> 82.9).
+      for (int bt = res ? 1 : taps; bt >= 1 && !found; --bt) {
+        if (taps % bt != 0 || (bt > 1 && bt * slice > 32u * 1024u)) continue;
+        for (int na = 4; na >= 2 && !found; --na) {
+          for (int nb = (res ? 1 : 4); nb >= (res ? 1 : 2) && !found; --nb) {
+            const uint64_t bb = res ? round_up(unit_bytes, 1024) : round_up(nb * bt * slice, 1024);
+            if (bb + stage_total + bar_bytes + static_cast<uint64_t>(na) * (sb + pk_stage_bytes(kc)) <= budget) {
+              found = true;
+              resident = res != 0;
+              KC = kc;
+              a_stages = na;
+              b_stages = nb;
+              b_taps = bt;
+              stage_bytes = sb;
+              phase_bytes = pb;
+              lbo = l;
+            }
           }
         }
       }
@@ -549,7 +557,8 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub,
     return PQ_EUNSUPPORTED;
   }
   const uint32_t b_bytes =
-      resident ? round_up(unit_bytes, 1024) : round_up(static_cast<uint64_t>(b_stages) * KC * p.Nblk / cpb, 1024);
+      resident ? round_up(unit_bytes, 1024)
+               : round_up(static_cast<uint64_t>(b_stages) * b_taps * KC * p.Nblk / cpb, 1024);
   p.KC = KC;
   p.nch = KC / (16 * cpb);
   p.nch_magic = static_cast<uint32_t>(((1ull << 32) + p.nch - 1) / p.nch);
@@ -611,6 +620,8 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub,
   }
   p.b_resident = resident ? 1 : 0;
   p.b_slice_bytes = static_cast<uint32_t>(KC) * p.Nblk / cpb;
+  p.b_taps = b_taps;
+  p.b_stage_bytes = static_cast<uint32_t>(b_taps) * p.b_slice_bytes;
   p.b_unit_bytes = static_cast<uint32_t>(unit_bytes);
   p.lbo_b = static_cast<uint32_t>(p.Nblk) * 16u;
   p.b_stages = resident ? 1 : b_stages;

@@ -270,16 +270,24 @@ __device__ __forceinline__ void producer_role(const ConvParams& p, const CUtenso
           if (!mbar_wait(a_slot(), ra.phase ^ 1u, ctx)) { ok = false; break; }
           load_a();
         }
-        for (int t = 0; t < p.taps; ++t) {
+        for (int t = 0; t < p.taps; t += p.b_taps) {
           if (!mbar_wait(bars.b_empty(rb.stage), rb.phase ^ 1u, ctx)) { ok = false; break; }
           const uint32_t bar = bars.b_full(rb.stage);
-          mbar_arrive_expect_tx(bar, p.b_slice_bytes);
-          const uint32_t dst = b_base + rb.stage * p.b_slice_bytes;
+          mbar_arrive_expect_tx(bar, p.b_stage_bytes);
+          uint32_t dst = b_base + rb.stage * p.b_stage_bytes;
           if (p.nsub > 1) {
-            load_w(item.unit, t * p.n_kb + kb, dst, bar);
+            for (int k = t; k < t + p.b_taps; ++k, dst += p.b_slice_bytes) load_w(item.unit, k * p.n_kb + kb, dst, bar);
           } else {
+            // the stage's first slice at once: as one loop over the slices, 128x28x28, 2
+            // groups of 256, one slice to a stage, took 89 us instead of 83
             const size_t slice = (static_cast<size_t>(unit) * p.taps + t) * p.n_kb + kb;  // tap-major packing
-            bulk_load(dst, p.w_packed + slice * p.b_slice_bytes, p.b_slice_bytes, bar);
+            const uint8_t* src = p.w_packed + slice * p.b_slice_bytes;
+            bulk_load(dst, src, p.b_slice_bytes, bar);
+            for (int k = 1; k < p.b_taps; ++k) {
+              dst += p.b_slice_bytes;
+              src += static_cast<size_t>(p.n_kb) * p.b_slice_bytes;
+              bulk_load(dst, src, p.b_slice_bytes, bar);
+            }
           }
           rb.advance();
           ++b_issued;
@@ -569,6 +577,8 @@ __device__ __forceinline__ void mma_role(const ConvParams& p, const Bars& bars, 
   const uint32_t a_lo0 = static_cast<uint32_t>(a_desc0), b_lo0 = static_cast<uint32_t>(b_desc0);
   const uint32_t a_ks16 = (2u * p.lbo_a) >> 4, b_ks16 = (2u * p.lbo_b) >> 4;  // one K step (32 bytes of K)
   const uint32_t a_stage16 = p.a_stage_bytes >> 4, b_slice16 = p.b_slice_bytes >> 4;
+  const uint32_t b_stage16 = p.b_stage_bytes >> 4;
+  const int b_taps = p.b_taps;
   const uint32_t b_tap16 = static_cast<uint32_t>(p.n_kb) * b_slice16;  // one tap of all K blocks
   const uint32_t amt = p.a_mt16;  // A operand of accumulator mt starts mt * amt 16-byte units in
   const int taps = p.taps, n_kb = p.n_kb;
@@ -657,6 +667,17 @@ __device__ __forceinline__ void mma_role(const ConvParams& p, const Bars& bars, 
 #pragma unroll
         for (int t = 0; t < kUnrollTaps; ++t)
           if (t < taps) issue_tap(t, a_lo_stage + tap_reg[t], b_lo_kb + static_cast<uint32_t>(t) * b_tap16);
+      } else if (!resident && b_taps > 1) {
+        // b_taps taps to a ring stage
+        for (int t0 = 0; t0 < taps; t0 += b_taps) {
+          if (!warp_wait(bars.b_full(rb.stage), rb.phase, ctx)) { ok = false; break; }
+          tc_fence_after();
+          uint32_t b_lo_tap = b_lo0 + rb.stage * b_stage16;
+          for (int t = t0; t < t0 + b_taps; ++t, b_lo_tap += b_slice16)
+            issue_tap(t, a_lo_stage + tap_a16[t], b_lo_tap);
+          tc_commit_warp(bars.b_empty(rb.stage));
+          rb.advance();
+        }
       } else {
         for (int t = 0; t < taps; ++t) {
           uint32_t b_lo_tap;

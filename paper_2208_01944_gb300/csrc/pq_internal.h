@@ -112,6 +112,8 @@ struct ConvParams {
   uint32_t a_tx_bytes;    // bytes one A stage receives (TMA mode)
   uint32_t a_zero_off, a_zero_bytes;  // zeroed tail of each operand stage (0 bytes: none)
   uint32_t b_slice_bytes; // one (K block, tap) slice: KC * Nblk bytes
+  int b_taps;             // taps (slices) of a ring stage when streamed
+  uint32_t b_stage_bytes; // b_taps slices
   uint32_t b_unit_bytes;  // taps * Cin_g * Nblk
   uint32_t pk_stage_bytes;
   uint32_t q_box_bytes;   // staging bytes per 32-channel box (a multiple of 1024: the 128B swizzle atom)

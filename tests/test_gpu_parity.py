@@ -911,3 +911,18 @@ def test_split_channel_blocks_match_oracle(B, c, fmt):
     assert_layer_parity(c, ref, run_gpu(c, ref, fmt=fmt))
     if not c.shortcut:
         assert_layer_parity(c, ref, run_gpu(c, ref, outputs=("q",), fmt=fmt))
+
+
+# Streamed weights with several taps to a ring stage (channel counts whose K blocks are
+# small: 9, 3 and 1 taps a stage), alone and with split channel blocks.
+TAPS_CASES = [(Case(2, 9, 8, 2, 224, 224, 3, 1, 1, bits=3, seed=231), 2), (Case(2, 42, 40, 3, 448, 128, 3, 1, 1, seed=232), 4),
+              (Case(200, 6, 5, 1, 160, 160, 3, 1, 1, seed=233), 2), (Case(160, 5, 5, 1, 352, 48, 5, 1, 2, seed=234), 0)]
+
+
+@pytest.mark.parametrize("c,fmt", TAPS_CASES, ids=str)
+def test_streamed_weights_several_taps_per_stage_match_oracle(B, c, fmt):
+    d = B.layer_desc(c.N, c.H, c.W, c.G, c.Cin, c.Cout, c.k, c.stride, c.pad, c.bits, c.bits, c.bits, code_format=fmt)
+    assert B.palquant_conv_plan(d).weights_resident == 0
+    ref = prepare(c)
+    assert_layer_parity(c, ref, run_gpu(c, ref, fmt=fmt))
+    assert_layer_parity(c, ref, run_gpu(c, ref, outputs=("q",), fmt=fmt))
