@@ -184,6 +184,14 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// ------------------------------------------------- programmatic dependent launch
+// Wait for the previous kernel on the stream (at once if this one was launched without
+// the attribute), then let the next dependent launch start its CTAs as SMs free up.  In
+// this order the kernels before the previous one have completed when that launch starts.
+__device__ __forceinline__ void pdl_wait_then_trigger() {
+  asm volatile("griddepcontrol.wait;\ngriddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ------------------------------------------------------------ packed fp32
 // Two IEEE fp32 round-to-nearest multiplies / adds in one instruction
 // (sm_100+ f32x2 arithmetic); lane-wise identical to __fmul_rn / __fadd_rn.

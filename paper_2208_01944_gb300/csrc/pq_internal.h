@@ -194,6 +194,28 @@ struct PwParams {
   int pdl, pdl_early_loads;
 };
 
+// Launch as a programmatic dependent of the previous kernel on the stream: the launch
+// itself overlaps that kernel's end.  The kernel calls pdl_wait_then_trigger() before its
+// first global access.  (The six launches of a layer's quantisers in training, 64x56x56,
+// 4 groups of 64: 205.7 us as plain launches, 193.5 so.  The inference quantisers stay
+// plain: their blocks, launched early beside a layer's CTAs, cost 20x37x45 NHWC 38.5 ->
+// 40.8 us.)
+template <typename... Params, typename... Args>
+inline cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                    Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // Host-side launch helpers implemented in the .cu files.
 int launch_conv_tc(const ConvParams& p, const CUtensorMap& tma_a, const CUtensorMap& tma_w, int grid,
                    cudaStream_t stream);

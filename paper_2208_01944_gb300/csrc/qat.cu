@@ -11,6 +11,7 @@
 #include <cstring>
 
 #include "palquant.h"
+#include "pq_device.cuh"
 #include "pq_internal.h"
 
 namespace pq {
@@ -71,6 +72,7 @@ __global__ void __launch_bounds__(kQatThreads) pq_fake_quant_fwd(const float4* _
   const int g = static_cast<int>(blockIdx.x % G);
   const uint32_t b = blockIdx.x / G, nb = gridDim.x / G;
   const float l = q.l[g], inv_r = q.inv_r[g];
+  pdl_wait_then_trigger();
   const uint32_t e0 = static_cast<uint32_t>(static_cast<uint64_t>(b) * q.quads / nb);
   const uint32_t e1 = static_cast<uint32_t>(static_cast<uint64_t>(b + 1) * q.quads / nb);
   // two float4s per thread and pass, both loads issued before either is used
@@ -114,6 +116,7 @@ __global__ void __launch_bounds__(kQatThreads, 8) pq_fake_quant_bwd(const float4
   const int g = static_cast<int>(blockIdx.x % G);
   const uint32_t b = blockIdx.x / G, nb = gridDim.x / G;
   const float l = q.l[g], u = q.u[g], inv_r = q.inv_r[g], k = q.k[g];
+  pdl_wait_then_trigger();
   const uint32_t e0 = static_cast<uint32_t>(static_cast<uint64_t>(b) * q.quads / nb);
   const uint32_t e1 = static_cast<uint32_t>(static_cast<uint64_t>(b + 1) * q.quads / nb);
   KahanF ka, kb;
@@ -176,6 +179,7 @@ __global__ void __launch_bounds__(kQatThreads) pq_fake_quant_bwd_finish(const do
                                                                         double* __restrict__ dl,
                                                                         double* __restrict__ du) {
   const int g = blockIdx.x;
+  pdl_wait_then_trigger();
   double sa = 0.0, sb = 0.0;
   for (int b = threadIdx.x; b < nblocks; b += kQatThreads) {
     const double2 v = partial[static_cast<int64_t>(g) * nblocks + b];
@@ -255,9 +259,10 @@ pq_status palquant_fake_quant_forward(const float* x_dev, float* xhat_dev, int64
   if (P == 0) return PQ_OK;  // no elements (the pointers may be NULL)
   if (x_dev == nullptr || xhat_dev == nullptr || !pq::aligned16(x_dev) || !pq::aligned16(xhat_dev)) return PQ_EINVAL;
   const unsigned grid = static_cast<unsigned>(pq::qat_blocks(q.quads)) * G;
-  pq::pq_fake_quant_fwd<<<grid, pq::kQatThreads, 0, static_cast<cudaStream_t>(stream)>>>(
-      reinterpret_cast<const float4*>(x_dev), reinterpret_cast<float4*>(xhat_dev), G, q);
-  return cudaGetLastError() == cudaSuccess ? PQ_OK : PQ_ECUDA;
+  const cudaError_t e =
+      pq::launch_dependent(pq::pq_fake_quant_fwd, grid, pq::kQatThreads, 0, static_cast<cudaStream_t>(stream),
+                           reinterpret_cast<const float4*>(x_dev), reinterpret_cast<float4*>(xhat_dev), G, q);
+  return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? PQ_OK : PQ_ECUDA;
 }
 
 size_t palquant_fake_quant_scratch_bytes(int64_t P, int32_t G, int32_t Cg) {
@@ -280,8 +285,9 @@ pq_status palquant_fake_quant_backward(const float* x_dev, const float* dy_dev, 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const double c = kind ? 2.0 : 1.0;
   if (P == 0) {  // no elements: zero gradients (the element pointers and the scratch may be NULL)
-    pq::pq_fake_quant_bwd_finish<<<G, pq::kQatThreads, 0, s>>>(nullptr, 0, c, q, dl_dev, du_dev);
-    return cudaGetLastError() == cudaSuccess ? PQ_OK : PQ_ECUDA;
+    const cudaError_t e =
+        pq::launch_dependent(pq::pq_fake_quant_bwd_finish, G, pq::kQatThreads, 0, s, nullptr, 0, c, q, dl_dev, du_dev);
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? PQ_OK : PQ_ECUDA;
   }
   if (x_dev == nullptr || dy_dev == nullptr || dx_dev == nullptr || scratch_dev == nullptr) return PQ_EINVAL;
   if (!pq::aligned16(x_dev) || !pq::aligned16(dy_dev) || !pq::aligned16(dx_dev) || !pq::aligned16(scratch_dev))
@@ -289,12 +295,12 @@ pq_status palquant_fake_quant_backward(const float* x_dev, const float* dy_dev, 
   if (scratch_bytes < palquant_fake_quant_scratch_bytes(P, G, Cg)) return PQ_EINVAL;
   const int nb = pq::qat_blocks(q.quads);
   double2* partial = static_cast<double2*>(scratch_dev);
-  pq::pq_fake_quant_bwd<<<static_cast<unsigned>(nb) * G, pq::kQatThreads, 0, s>>>(
-      reinterpret_cast<const float4*>(x_dev), reinterpret_cast<const float4*>(dy_dev),
-      reinterpret_cast<float4*>(dx_dev), partial, G, q);
-  if (cudaGetLastError() != cudaSuccess) return PQ_ECUDA;
-  pq::pq_fake_quant_bwd_finish<<<G, pq::kQatThreads, 0, s>>>(partial, nb, c, q, dl_dev, du_dev);
-  return cudaGetLastError() == cudaSuccess ? PQ_OK : PQ_ECUDA;
+  cudaError_t e = pq::launch_dependent(pq::pq_fake_quant_bwd, static_cast<unsigned>(nb) * G, pq::kQatThreads, 0, s,
+                                       reinterpret_cast<const float4*>(x_dev), reinterpret_cast<const float4*>(dy_dev),
+                                       reinterpret_cast<float4*>(dx_dev), partial, G, q);
+  if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) return PQ_ECUDA;
+  e = pq::launch_dependent(pq::pq_fake_quant_bwd_finish, G, pq::kQatThreads, 0, s, partial, nb, c, q, dl_dev, du_dev);
+  return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? PQ_OK : PQ_ECUDA;
 }
 
 }  // extern "C"
