@@ -342,11 +342,16 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub,
     }
     // Few items for the chip: the longest CTA's time counts, in whole items, and a block
     // of output channels may be split between CTAs (each loads its columns of the packed
-    // weights).  Each item costs as above, with the general epilogue's units at 1500 ns
+    // weights).  Each item costs as above, with the general epilogue's units at 2000 ns
     // (32 columns) or 850; the weights that stay are loaded once, streamed ones for every
-    // item, at 80 B/ns; the shorter of the MMAs and the epilogue is paid once more.  The
-    // network at batch 1 (8 to 20 items a layer before): 218 -> 197 us.  A layer that the
-    // rule above cannot plan stays refused, and keeps that plan where this one has none.
+    // item, at 80 B/ns; the shorter of the MMAs and the epilogue is paid once more; a
+    // split costs 1200 ns (a second tensor map, a load per slice) and a CTA 8 ns.  The
+    // network at batch 1 (8 to 20 items a layer before): 218 -> 197 us, and 169 -> 166
+    // with the last two terms (4 images of 14x14, 2 groups of 256, codes only: 6.1 -> 5.0
+    // us; general 9.0 -> 7.6).  One image, codes only / with shortcut and fp32 out, without
+    // and with this rule: 56x56, 2 groups of 64, 4.3 -> 3.7 / 8.7 -> 5.9 us; 7x7, 2 groups
+    // of 512, 6.6 -> 6.0 / 9.8 -> 9.0 us.  A layer that the rule above cannot plan stays
+    // refused, and keeps that plan where this one has none.
     if (items_of(best) < 8 * kPlanSMs && d->N > 0) {
       Tile fast;
       const int64_t items0 = items_of(best);
@@ -359,7 +364,7 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub,
           if (!tile_of(MT, n_cols, &t)) continue;
           const bool wide = direct_out ? f4 && n_cols % 32 == 0 : n_cols % 32 == 0;  // 32-column units
           const int units = MT * n_cols / (wide ? 32 : 16);
-          const double u_ns = direct_out ? (wide ? 550.0 : 430.0) : (wide ? 1500.0 : 850.0);
+          const double u_ns = direct_out ? (wide ? 550.0 : 430.0) : (wide ? 2000.0 : 850.0);
           const double epi = ((units + epi_groups - 1) / epi_groups) * u_ns;
           const int np2 = next_pow2(n_cols);
           const double w_bytes = static_cast<double>(taps) * d->Cin_g * n_cols / cpb;
@@ -369,7 +374,8 @@ pq_status plan_conv(const pq_layer_desc* d, ConvParams* P, pq_conv_plan* pub,
                                       stream ? w_bytes / 80.0 : 0.0);
           const int64_t waves = (items_of(t) + kPlanSMs - 1) / kPlanSMs;
           const double item_ns = 500.0 + (t.acc_stages == 1 && waves > 1 ? mma + epi : std::max(mma, epi));
-          t.cost = (stream ? 0.0 : w_bytes / 80.0) + waves * item_ns + std::min(mma, epi);
+          t.cost = (stream ? 0.0 : w_bytes / 80.0) + waves * item_ns + std::min(mma, epi) + (nsub > 1 ? 1200.0 : 0.0) +
+                   8.0 * static_cast<double>(std::min<int64_t>(items_of(t), kPlanSMs));
           if (fast.MT == 0 || t.cost < fast.cost * 0.97) fast = t;
         }
       }
