@@ -926,3 +926,15 @@ def test_streamed_weights_several_taps_per_stage_match_oracle(B, c, fmt):
     ref = prepare(c)
     assert_layer_parity(c, ref, run_gpu(c, ref, fmt=fmt))
     assert_layer_parity(c, ref, run_gpu(c, ref, outputs=("q",), fmt=fmt))
+
+
+# Resident weights with three operand stages' room, which two MMA warps share as two
+# (128 byte channels, 256 FP4 channels); the last has more taps than are unrolled.
+@pytest.mark.parametrize("c,fmt", [(Case(44, 28, 28, 4, 128, 128, 3, 1, 1, bits=3, seed=241), 2),
+                                   (Case(45, 28, 28, 2, 256, 256, 3, 1, 1, seed=242), 4),
+                                   (Case(50, 20, 20, 2, 64, 64, 5, 1, 2, seed=243), 2)], ids=str)
+def test_resident_weights_ring_codes_only_match_oracle(B, c, fmt):
+    d = B.layer_desc(c.N, c.H, c.W, c.G, c.Cin, c.Cout, c.k, c.stride, c.pad, c.bits, c.bits, c.bits, code_format=fmt)
+    assert B.palquant_conv_plan(d).weights_resident == 1
+    ref = prepare(c)
+    assert_layer_parity(c, ref, run_gpu(c, ref, outputs=("q",), fmt=fmt))
