@@ -580,6 +580,7 @@ __device__ __forceinline__ void mma_role(const ConvParams& p, const Bars& bars, 
   const uint32_t b_stage16 = p.b_stage_bytes >> 4;
   const int b_taps = p.b_taps;
   const uint32_t b_tap16 = static_cast<uint32_t>(p.n_kb) * b_slice16;  // one tap of all K blocks
+  const uint32_t b_step16 = p.b_resident ? b_tap16 : b_slice16;  // from a tap to the next
   const uint32_t amt = p.a_mt16;  // A operand of accumulator mt starts mt * amt 16-byte units in
   const int taps = p.taps, n_kb = p.n_kb;
   const uint32_t npow2 = static_cast<uint32_t>(p.Npow2);
@@ -667,32 +668,34 @@ __device__ __forceinline__ void mma_role(const ConvParams& p, const Bars& bars, 
 #pragma unroll
         for (int t = 0; t < kUnrollTaps; ++t)
           if (t < taps) issue_tap(t, a_lo_stage + tap_reg[t], b_lo_kb + static_cast<uint32_t>(t) * b_tap16);
-      } else if (!resident && b_taps > 1) {
-        // b_taps taps to a ring stage
-        for (int t0 = 0; t0 < taps; t0 += b_taps) {
-          if (!warp_wait(bars.b_full(rb.stage), rb.phase, ctx)) { ok = false; break; }
-          tc_fence_after();
-          uint32_t b_lo_tap = b_lo0 + rb.stage * b_stage16;
-          for (int t = t0; t < t0 + b_taps; ++t, b_lo_tap += b_slice16)
-            issue_tap(t, a_lo_stage + tap_a16[t], b_lo_tap);
-          tc_commit_warp(bars.b_empty(rb.stage));
-          rb.advance();
-        }
-      } else {
-        for (int t = 0; t < taps; ++t) {
-          uint32_t b_lo_tap;
-          if (resident) {
-            b_lo_tap = b_lo_kb + static_cast<uint32_t>(t) * b_tap16;
-          } else {
+      } else if (resident || b_taps > 1) {
+        // b_taps taps to a ring stage; resident weights of more than 9 taps as one run (5x5,
+        // 195x20x20, 4 groups of 64 byte codes: 40.8 us with the loop below, 37.1 here)
+        const int step = resident ? taps : b_taps;
+        for (int t0 = 0; t0 < taps; t0 += step) {
+          uint32_t b_lo_tap = b_lo_kb;
+          if (!resident) {
             if (!warp_wait(bars.b_full(rb.stage), rb.phase, ctx)) { ok = false; break; }
             tc_fence_after();
-            b_lo_tap = b_lo0 + rb.stage * b_slice16;
+            b_lo_tap = b_lo0 + rb.stage * b_stage16;
           }
-          issue_tap(t, a_lo_stage + tap_a16[t], b_lo_tap);
+#pragma unroll 1
+          for (int t = t0; t < t0 + step; ++t, b_lo_tap += b_step16)
+            issue_tap(t, a_lo_stage + tap_a16[t], b_lo_tap);
           if (!resident) {
             tc_commit_warp(bars.b_empty(rb.stage));
             rb.advance();
           }
+        }
+      } else {
+        // one slice to a stage, without the loop over a stage's taps (5x5, 66x28x28, 4
+        // groups of 96 byte codes: 55.8 us, 66.6 as a run of one tap)
+        for (int t = 0; t < taps; ++t) {
+          if (!warp_wait(bars.b_full(rb.stage), rb.phase, ctx)) { ok = false; break; }
+          tc_fence_after();
+          issue_tap(t, a_lo_stage + tap_a16[t], b_lo0 + rb.stage * b_slice16);
+          tc_commit_warp(bars.b_empty(rb.stage));
+          rb.advance();
         }
       }
       if (!ok) break;
