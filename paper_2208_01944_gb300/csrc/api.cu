@@ -1107,7 +1107,15 @@ pq_status layer_fused_impl(const void* q_dev, const void* w_packed_dev, const pq
   const int grid = static_cast<int>(std::min<int64_t>(sms, p.items));
   if (grid <= 0) return PQ_OK;
   p.items_per_cta = p.items / grid;
-  p.items_rem = p.items % grid;
+  p.items_rem = static_cast<int>(p.items % grid);
+  // The CTAs with an item more: spread over the grid where they are many (neighbouring SMs
+  // then seldom both run late), else the first ones, which start first.  Back to back,
+  // first / spread, by the share of such CTAs: 0.79 (64x56x56, 4 groups of 64, fp32 in, 1792
+  // items on 152 SMs: 50.9 / 49.7 us), 0.58 (128x28x28, 4 groups of 128: 42.8 / 41.9),
+  // 0.47 (128x28x28, 8 groups of 64: 37.7 / 36.5), 0.42 (99x14x15, 4 groups of 256, FP4:
+  // 20.2 / 21.1), 0.13 (390x20x20, 2 groups of 64: 17.9 / 18.7).  With streamed weights
+  // spreading only lost (7x7, 2 groups of 512, FP4: 20.0 / 20.9).
+  p.items_spread = p.b_resident && 16 * p.items_rem >= 7 * grid ? 1 : 0;
   CUtensorMap map;
   std::memset(&map, 0, sizeof(map));
   p.pdl = 1;  // programmatic dependent launch: the set-up overlaps the previous grid's last CTAs

@@ -1596,9 +1596,11 @@ __global__ void __launch_bounds__(kConvThreads, 1)
   // weights, pdl_early_loads) and the epilogue warps, which make every global store.
   // The MMA, quantiser, split and unpack roles work in shared and tensor memory only.
   // a contiguous range of items, sizes differing by at most one
-  const int64_t bx = static_cast<int64_t>(blockIdx.x);
-  const int64_t it0 = bx * p.items_per_cta + min(bx, p.items_rem);
-  const int64_t it1 = it0 + p.items_per_cta + (bx < p.items_rem ? 1 : 0);
+  const uint32_t bx = blockIdx.x, rem = static_cast<uint32_t>(p.items_rem);
+  const uint32_t x0 = p.items_spread ? bx * rem / gridDim.x : min(bx, rem);
+  const uint32_t x1 = p.items_spread ? (bx + 1) * rem / gridDim.x : min(bx + 1, rem);
+  const int64_t it0 = static_cast<int64_t>(bx) * p.items_per_cta + x0;
+  const int64_t it1 = it0 + p.items_per_cta + (x1 - x0);
   const uint32_t a_base = base;
   const uint32_t b_base = base + p.smem_b_off;
 

@@ -65,7 +65,9 @@ struct ConvParams {
   int img_pix;            // H * W (flat mode tiles stay inside one image)
   int64_t tiles;          // tiles per (group, n-block) unit
   int64_t items;          // tiles * G * NB
-  int64_t items_per_cta, items_rem;  // items / grid and items % grid: the first items_rem CTAs take one more
+  int64_t items_per_cta;  // items / grid
+  int items_rem;          // items % grid: this many CTAs take one more,
+  int items_spread;       // 1: evenly over the grid, 0: the first of it
   // pdl = 1: launched as a programmatic dependent of the previous kernel on the
   // stream: a CTA's set-up (barriers, tensor memory) may run while that kernel's
   // last CTAs still run; every global access waits for it to complete (stream
