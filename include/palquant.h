@@ -496,11 +496,13 @@ pq_status palquant_fake_quant_backward(const float* x_dev, const float* dy_dev, 
 typedef struct {
     int32_t supported;     /* 1 if the tensor-core kernel runs this layer */
     int32_t mode;          /* 0 flat pixels (1x1, stride 1, pad 0), 1 rows of whole image rows */
-    int32_t rows_per_tile; /* output rows per tile (mode 1) */
+    int32_t rows_per_tile; /* output rows per tile (mode 1); a tile may hold several small
+                              images, with that many rows of each */
     int32_t m_tiles;       /* 128-row accumulators per tile */
     int32_t tile_pitch;    /* positions per tile row in shared memory */
-    int32_t n_block;       /* output channels per accumulator (MMA N) */
-    int32_t n_blocks;      /* output-channel blocks per group */
+    int32_t n_block;       /* output channels per accumulator (MMA N); where a layer has few
+                              tiles, a part of a block of the packed weights */
+    int32_t n_blocks;      /* such blocks per group */
     int32_t k_chunk;       /* input channels per K block */
     int32_t k_blocks;      /* K blocks per tap */
     int32_t taps;          /* kh*kw */

@@ -8,17 +8,19 @@
 //   y = (float)acc * m_out[g] (+ shortcut) (ReLU);  q' = clamp(rint(t * m_req[g]), 0, Qp)
 // all written at the destination channel of (g, co).
 //
-// How (one persistent CTA per SM, warp-specialised):
-//  * warps 2-5 copy, per tile, the activation codes the tile needs with 16-byte
-//    cp.async straight into the tensor core's no-swizzle K-major operand layout:
-//    for each 16-byte chunk of input channels a plane of consecutive positions,
-//    one position per 16-byte row.  A "position" is a pixel of the zero-padded
-//    input tile (rows mode) or a pixel of the flattened batch (flat mode, 1x1
-//    layers).  Out-of-range pixels are zero-filled, which is exactly the zero
-//    padding (code 0).  Stride-2 layers get one plane set per stride phase of
-//    the input, so every tap is again a contiguous run of positions.  (A TMA box
-//    with a 16-byte inner extent moves one element per several cycles per SM and
-//    starved the tensor core; the LSU path moves 512 bytes per warp instruction.)
+// How (one persistent CTA per SM, 15 warps, warp-specialised):
+//  * the A operand is the tensor core's no-swizzle K-major layout: for each 16-byte
+//    chunk of input channels a plane of consecutive positions, one position per
+//    16-byte row.  A "position" is a pixel of the zero-padded input tile (rows mode;
+//    several whole images where they are small) or a pixel of the flattened image
+//    (flat mode, 1x1 layers).  Out-of-range pixels are zero-filled, which is exactly
+//    the zero padding (code 0).  Stride-2 layers get one plane set per stride phase of
+//    the input, so every tap is again a contiguous run of positions.
+//  * warp 0 loads channel-blocked codes by TMA, and the weights.  Warps 2-5 fill the
+//    operand stages where TMA alone cannot: NHWC codes with 16-byte cp.async (a TMA
+//    box with a 16-byte inner extent moves one element per several cycles and starved
+//    the tensor core), a stride-2 window split into its phases, packed codes unpacked,
+//    fp32 inputs quantised.  Else they are a third epilogue warpgroup.
 //  * The int8 codes are NOT converted: a byte v <= 15 is the FP8 E4M3 encoding of
 //    v * 2^-9 (subnormal and first binade are linear), so the tensor core reads
 //    the codes in place and every product and sum is exact in the fp32
@@ -27,15 +29,16 @@
 //    same layout; warp 0 bulk-copies them (cp.async.bulk) so they either stay
 //    resident in shared memory for the CTA's whole (group, output-block) unit or
 //    stream through a ring of (K block, tap) slices.
-//  * warp 1 (one lane) issues tcgen05.mma kind::f8f6f4 (M = 128, N = the output
-//    block): for every tap the A operand is the same planes with the start
-//    address moved by the tap's position offset (16 bytes per position), so a
-//    3x3 convolution needs no im2col copy.  Accumulators live in tensor memory,
-//    double-buffered so the epilogue of tile i overlaps the MMAs of tile i+1.
-//  * warps 6-13 (two warpgroups, each taking half of the output columns) read the
-//    accumulators (tcgen05.ld), apply the rescale, shortcut,
-//    ReLU, output permutation and requantisation in registers, stage rows in
-//    shared memory and write them with coalesced 16-byte stores.
+//  * warp 1 issues tcgen05.mma kind::f8f6f4, or kind::mxf4 for FP4 codes (M = 128,
+//    N = the output block): for every tap the A operand is the same planes with the
+//    start address moved by the tap's position offset (16 bytes per position), so a
+//    3x3 convolution needs no im2col copy.  Warp 14 takes every other item where the
+//    rings allow it (mma_role).  Accumulators live in tensor memory, double-buffered
+//    so the epilogue of tile i overlaps the MMAs of tile i+1.
+//  * warps 6-13 (two warpgroups, with warps 2-5 three) read the accumulators
+//    (tcgen05.ld) and apply the rescale, shortcut, ReLU, output permutation and
+//    requantisation in registers.  Channel-blocked codes are stored from registers,
+//    everything else as whole rows through a staging buffer per warp.
 //  * every wait is bounded (failure detection): a wait that runs out records
 //    PQ_ERR_TIMEOUT in the device error word, raises a CTA-wide abort flag, and
 //    every role drains what it has in flight and returns.
@@ -536,7 +539,7 @@ __device__ __forceinline__ void split_role(const ConvParams& p, const Bars& bars
 }
 
 // --------------------------------------------------------------------------
-// Tensor-core issue role (warp 1).
+// Tensor-core issue role (warps 1 and 14).
 // --------------------------------------------------------------------------
 
 constexpr int kUnrollTaps = 9;
@@ -736,7 +739,7 @@ __device__ __forceinline__ void mma_role_dispatch(const ConvParams& p, const Bar
 }
 
 // --------------------------------------------------------------------------
-// Epilogue role (warps 2-5).
+// Epilogue role (warps 6-13, and 2-5 under plain TMA loads).
 // --------------------------------------------------------------------------
 // Requantised code of t = clamp(rint(t), 0, qmax) with round-half-to-even, on the
 // FMA and integer pipes: clamping t to [-1, qmax + 1] first does not change the
