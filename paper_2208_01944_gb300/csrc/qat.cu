@@ -207,16 +207,19 @@ __global__ void __launch_bounds__(kQatThreads) pq_fake_quant_bwd_finish(const do
 // benchmark sizes; up to 64 blocks with one pass of two float4s each, where a group is too
 // small for that (the weights of 4 groups of 64x64x3x3: 18 blocks a group instead of 5,
 // so that its loads wait for memory once and not four times; with their activations,
-// 64x56x56, 193.5 -> 186.6 us).  Fixed by the problem size
-// only, so the partition, and the sums, do not depend on the device.
+// 64x56x56, 193.5 -> 186.6 us).  Fixed by the problem size only, so the partition, and the
+// sums, do not depend on the device.
+constexpr uint64_t kQatPass = kQatThreads * 2u;  // float4s of a block's pass
+
+int qat_blocks_deep(uint32_t quads) {
+  const uint64_t nb = (static_cast<uint64_t>(quads) + 4 * kQatPass - 1) / (4 * kQatPass);
+  return static_cast<int>(nb < 1 ? 1 : nb > kQatMaxBlocks ? kQatMaxBlocks : nb);
+}
+
 int qat_blocks(uint32_t quads) {
-  const uint64_t pass = kQatThreads * 2u;
-  uint64_t nb = (static_cast<uint64_t>(quads) + 4 * pass - 1) / (4 * pass);
-  const uint64_t one_pass = (static_cast<uint64_t>(quads) + pass - 1) / pass;
-  if (nb < 64) nb = one_pass < 64 ? one_pass : 64;
-  if (nb < 1) nb = 1;
-  if (nb > kQatMaxBlocks) nb = kQatMaxBlocks;
-  return static_cast<int>(nb);
+  const int nb = qat_blocks_deep(quads);
+  const uint64_t one_pass = (static_cast<uint64_t>(quads) + kQatPass - 1) / kQatPass;
+  return nb >= 64 ? nb : one_pass < 1 ? 1 : one_pass < 64 ? static_cast<int>(one_pass) : 64;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -298,8 +301,11 @@ pq_status palquant_fake_quant_backward(const float* x_dev, const float* dy_dev, 
   if (x_dev == nullptr || dy_dev == nullptr || dx_dev == nullptr || scratch_dev == nullptr) return PQ_EINVAL;
   if (!pq::aligned16(x_dev) || !pq::aligned16(dy_dev) || !pq::aligned16(dx_dev) || !pq::aligned16(scratch_dev))
     return PQ_EINVAL;
-  if (scratch_bytes < palquant_fake_quant_scratch_bytes(P, G, Cg)) return PQ_EINVAL;
-  const int nb = pq::qat_blocks(q.quads);
+  // Less scratch than palquant_fake_quant_scratch_bytes does for fewer, deeper blocks.
+  const size_t per_block = sizeof(double2) * static_cast<size_t>(G);
+  int nb = pq::qat_blocks(q.quads);
+  if (scratch_bytes < per_block * nb) nb = pq::qat_blocks_deep(q.quads);
+  if (scratch_bytes < per_block * nb) return PQ_EINVAL;
   double2* partial = static_cast<double2*>(scratch_dev);
   cudaError_t e = pq::launch_dependent(pq::pq_fake_quant_bwd, static_cast<unsigned>(nb) * G, pq::kQatThreads, 0, s,
                                        reinterpret_cast<const float4*>(x_dev), reinterpret_cast<const float4*>(dy_dev),

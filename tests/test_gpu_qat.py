@@ -56,7 +56,7 @@ CASES = [  # P, G, Cg, bits, kind
 ]
 
 
-def _run(B, x, dy, G, bits, kind, l, u):
+def _run(B, x, dy, G, bits, kind, l, u, sb=None):
     P, C = x.shape
     Cg = C // G
     xd = torch.from_numpy(x).cuda()
@@ -66,7 +66,7 @@ def _run(B, x, dy, G, bits, kind, l, u):
     dxd = torch.full_like(xd, 7.0)
     dl = torch.full((G,), 7.0, dtype=torch.float64, device="cuda")
     du = torch.full((G,), 7.0, dtype=torch.float64, device="cuda")
-    sb = B.palquant_fake_quant_scratch_bytes(P, G, Cg)
+    sb = B.palquant_fake_quant_scratch_bytes(P, G, Cg) if sb is None else sb
     scratch = torch.empty(max(sb, 16), dtype=torch.uint8, device="cuda")
     B.palquant_fake_quant_backward(xd, dyd, dxd, dl, du, P, G, Cg, bits, kind, l, u, scratch, sb)
     torch.cuda.synchronize()
@@ -125,3 +125,17 @@ def test_fake_quant_full_size_activations(B):
     assert np.array_equal(dx, dx_ref)
     bl, bu = _grad_bound(x, dy, G, 0, l, u, dx_ref)
     assert np.all(np.abs(dl - dl_ref) <= bl) and np.all(np.abs(du - du_ref) <= bu)
+
+
+def test_fake_quant_backward_with_scratch_for_eight_float4s_a_thread(B):
+    # 16000 float4s a group: 8 blocks of 256 threads with eight float4s each, 16 bytes a
+    # block and group, instead of one pass of two float4s; less than that is refused
+    x, dy, l, u = _inputs(1000, 4, 64, 2, seed=4)
+    assert B.palquant_fake_quant_scratch_bytes(1000, 4, 64) > 8 * 4 * 16
+    _, dx, dl, du = _run(B, x, dy, 4, 2, 0, l, u, sb=8 * 4 * 16)
+    dx_ref, dl_ref, du_ref = oracle.fake_quant_backward(x, dy, 4, 2, 0, l, u)
+    bl, bu = _grad_bound(x, dy, 4, 0, l, u, dx_ref)
+    assert np.array_equal(dx, dx_ref, equal_nan=True)
+    assert np.all(np.abs(dl - dl_ref) <= bl) and np.all(np.abs(du - du_ref) <= bu)
+    with pytest.raises(B.PalquantError):
+        _run(B, x, dy, 4, 2, 0, l, u, sb=8 * 4 * 16 - 16)
