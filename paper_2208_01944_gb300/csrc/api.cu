@@ -1114,8 +1114,10 @@ pq_status layer_fused_impl(const void* q_dev, const void* w_packed_dev, const pq
   // items on 152 SMs: 50.9 / 49.7 us), 0.58 (128x28x28, 4 groups of 128: 42.8 / 41.9),
   // 0.47 (128x28x28, 8 groups of 64: 37.7 / 36.5), 0.42 (99x14x15, 4 groups of 256, FP4:
   // 20.2 / 21.1), 0.13 (390x20x20, 2 groups of 64: 17.9 / 18.7).  With streamed weights
-  // spreading only lost (7x7, 2 groups of 512, FP4: 20.0 / 20.9).
-  p.items_spread = p.b_resident && 16 * p.items_rem >= 7 * grid ? 1 : 0;
+  // spreading only lost (7x7, 2 groups of 512, FP4: 20.0 / 20.9), and so it did where loads
+  // start before the previous launch ends: CTAs then start as SMs free up, the first ones
+  // well ahead (fp32 in, as above: 46.7 / 47.5; 8 groups of 64: 35.0 / 36.8).
+  p.items_spread = p.b_resident && (d->flags & PQ_LAYER_INPUTS_READY) == 0 && 16 * p.items_rem >= 7 * grid ? 1 : 0;
   CUtensorMap map;
   std::memset(&map, 0, sizeof(map));
   p.pdl = 1;  // programmatic dependent launch: the set-up overlaps the previous grid's last CTAs
