@@ -967,9 +967,10 @@ __device__ __forceinline__ void quant_role(const ConvParams& p, const Bars& bars
 // code 0.
 //
 // Instruction fetch bounds these units before memory does (the largest stall of the
-// 128x56x56 layer with shortcut when a unit took 900 instructions), so addresses are a
-// 64-bit base per item plus a 32-bit pixel times the row's bytes, a row's entry is
-// computed when the accumulator changes, and units advance without divisions.
+// 56x56 layer with shortcut, 2 groups of 64), so addresses are a 64-bit base per item plus
+// a 32-bit pixel times the row's bytes, a row's entry is computed when the accumulator
+// changes, and units advance without divisions: a launch of 48 images executes 16.9 M
+// instructions instead of 20.7 M, one of 128 takes 83 us instead of 101.
 template <int UC>
 __device__ __forceinline__ uint32_t row_swizzle(int r) {
   constexpr int CPR = UC / 4;  // 16-byte chunks per staged row
