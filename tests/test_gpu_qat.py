@@ -56,7 +56,7 @@ CASES = [  # P, G, Cg, bits, kind
 ]
 
 
-def _run(B, x, dy, G, bits, kind, l, u, sb=None):
+def _run(B, x, dy, G, bits, kind, l, u):
     P, C = x.shape
     Cg = C // G
     xd = torch.from_numpy(x).cuda()
@@ -66,7 +66,7 @@ def _run(B, x, dy, G, bits, kind, l, u, sb=None):
     dxd = torch.full_like(xd, 7.0)
     dl = torch.full((G,), 7.0, dtype=torch.float64, device="cuda")
     du = torch.full((G,), 7.0, dtype=torch.float64, device="cuda")
-    sb = B.palquant_fake_quant_scratch_bytes(P, G, Cg) if sb is None else sb
+    sb = B.palquant_fake_quant_scratch_bytes(P, G, Cg)
     scratch = torch.empty(max(sb, 16), dtype=torch.uint8, device="cuda")
     B.palquant_fake_quant_backward(xd, dyd, dxd, dl, du, P, G, Cg, bits, kind, l, u, scratch, sb)
     torch.cuda.synchronize()
@@ -130,12 +130,18 @@ def test_fake_quant_full_size_activations(B):
 def test_fake_quant_backward_with_scratch_for_eight_float4s_a_thread(B):
     # 16000 float4s a group: 8 blocks of 256 threads with eight float4s each, 16 bytes a
     # block and group, instead of one pass of two float4s; less than that is refused
-    x, dy, l, u = _inputs(1000, 4, 64, 2, seed=4)
-    assert B.palquant_fake_quant_scratch_bytes(1000, 4, 64) > 8 * 4 * 16
-    _, dx, dl, du = _run(B, x, dy, 4, 2, 0, l, u, sb=8 * 4 * 16)
-    dx_ref, dl_ref, du_ref = oracle.fake_quant_backward(x, dy, 4, 2, 0, l, u)
-    bl, bu = _grad_bound(x, dy, 4, 0, l, u, dx_ref)
-    assert np.array_equal(dx, dx_ref, equal_nan=True)
-    assert np.all(np.abs(dl - dl_ref) <= bl) and np.all(np.abs(du - du_ref) <= bu)
+    P, G, Cg, sb = 1000, 4, 64, 8 * 4 * 16
+    x, dy, l, u = _inputs(P, G, Cg, 2, seed=4)
+    assert B.palquant_fake_quant_scratch_bytes(P, G, Cg) > sb
+    xd, dyd = torch.from_numpy(x).cuda(), torch.from_numpy(dy).cuda()
+    dxd = torch.full_like(xd, 7.0)
+    dl, du = (torch.full((G,), 7.0, dtype=torch.float64, device="cuda") for _ in range(2))
+    scratch = torch.empty(sb, dtype=torch.uint8, device="cuda")
     with pytest.raises(B.PalquantError):
-        _run(B, x, dy, 4, 2, 0, l, u, sb=8 * 4 * 16 - 16)
+        B.palquant_fake_quant_backward(xd, dyd, dxd, dl, du, P, G, Cg, 2, 0, l, u, scratch, sb - 16)
+    B.palquant_fake_quant_backward(xd, dyd, dxd, dl, du, P, G, Cg, 2, 0, l, u, scratch, sb)
+    torch.cuda.synchronize()
+    dx_ref, dl_ref, du_ref = oracle.fake_quant_backward(x, dy, G, 2, 0, l, u)
+    bl, bu = _grad_bound(x, dy, G, 0, l, u, dx_ref)
+    assert np.array_equal(dxd.cpu().numpy(), dx_ref, equal_nan=True)
+    assert np.all(np.abs(dl.cpu().numpy() - dl_ref) <= bl) and np.all(np.abs(du.cpu().numpy() - du_ref) <= bu)
